@@ -5,10 +5,12 @@
 // Three kernels.  reinsert_kernel runs one scenario per warp (the two
 // actions), reinsert_routes_kernel one scenario per warp with up to K route
 // options, and reinsert_lane_kernel (below) one scenario per lane, for the
-// two actions or up to 8 route options.  SDP_REINSERT_AUTO takes the lane
-// kernel wherever it applies (U <= 255, T <= 4096, at least 4 warps' worth of
-// its shared memory per SM; not with a table end cost and route options);
-// SDP_REINSERT_WARP forces the warp kernels.
+// two actions or up to 8 route options.  All three evaluate every state of
+// every day; SDP_REINSERT_AUTO takes reinsert_chain.cu's kernel, over the
+// reachable states only, where it applies and C_0(I) is not wanted for every
+// I, else the lane kernel wherever it applies (U <= 255, T <= 4096, at least 4
+// warps' worth of its shared memory per SM; not with a table end cost and
+// route options).  SDP_REINSERT_WARP forces the warp kernels.
 //
 // Mapping of the warp kernels.  One warp per scenario; lane l owns the inventory states
 // I = l + 32k, k < KC, so the consumption of the day is warp-uniform and the
@@ -808,6 +810,9 @@ size_t reinsert_lane_scratch_bytes(int T, int U) {
 
 int launch_reinsert(const ReinsertArgs& a, cudaStream_t st) {
   if (a.S <= 0) return 0;
+  if (a.algo == SDP_REINSERT_AUTO && !a.value0 &&
+      reinsert_chain_supported(a.T, a.U, a.table != nullptr, a.n_routes, a.h, a.p, a.c))
+    return launch_reinsert_chain(a, st);
   const bool unit = a.c != 0.f;
   if (a.n_routes > 0) {  // route options: U <= 255, linear end costs (checked by the caller)
     if (a.U > 255 || a.table) return (int)cudaErrorInvalidValue;
@@ -820,7 +825,7 @@ int launch_reinsert(const ReinsertArgs& a, cudaStream_t st) {
     }
     return unit ? routes_by_kc<true>(a, st) : routes_by_kc<false>(a, st);
   }
-  // AUTO takes LANE where it applies: at T = 60, U = 200, S = 10^6 it runs in
+  // else AUTO takes LANE where it applies: at T = 60, U = 200, S = 10^6 it runs in
   // 5.20 ms against 6.17 ms for WARP (a register-resident variant of WARP,
   // shifting the cost-to-go by warp shuffles, was measured at 6.59 ms: a
   // shuffle and a select cost what the shared load and store they replace

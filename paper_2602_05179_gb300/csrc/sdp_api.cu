@@ -985,6 +985,9 @@ namespace {
 // the lane kernel keeps its decision bits in the workspace when the policy
 // is wanted
 bool reinsert_uses_lane(const sdp_reinsert_args* a) {
+  if (a->algo == SDP_REINSERT_AUTO && !a->value0_out &&
+      reinsert_chain_supported(a->T, a->U, a->end_cost_table != nullptr, a->n_routes, a->h, a->p, a->unit_cost))
+    return false;
   return (a->algo == SDP_REINSERT_LANE || a->algo == SDP_REINSERT_AUTO) &&
          !(a->n_routes > 0 && a->end_cost_table) &&
          reinsert_lane_supported(a->T, a->U, a->n_routes);

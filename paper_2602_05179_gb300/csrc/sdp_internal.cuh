@@ -388,6 +388,9 @@ size_t reinsert_lane_smem(int T, int U, bool table);
 size_t reinsert_lane_smem_for(int T, int U, bool table, int warps, int n_routes);
 int reinsert_lane_warps(int T, int U, bool table, int n_routes);
 size_t reinsert_lane_scratch_bytes(int T, int U);
+// the states reachable from I0 only (reinsert_chain.cu): AUTO without value0
+bool reinsert_chain_supported(int T, int U, bool table, int n_routes, float h, float p, float c);
+int launch_reinsert_chain(const ReinsertArgs& a, cudaStream_t st);
 
 int num_sms();
 
