@@ -807,9 +807,11 @@ FleetWs carve_fleet(const sdp_split_args* a, int K, bool routes, void* base) {
   const int64_t cap = plain ? kFleetPlainSlots : kFleetFallbackSlots;
   w.nslots = a->S < cap ? a->S : cap;
   if (w.nslots < 1) w.nslots = 1;
-  w.kscratch = c.take<float>((size_t)w.nslots * 2 * (size_t)(n + 1));
-  w.pscratch = routes ? c.take<uint16_t>((size_t)w.nslots * K * (size_t)n) : nullptr;
   w.cfg = plain || n == 0 ? FleetConfig{} : fleet_config(n, K, a->S);
+  if (!w.cfg.band) {
+    w.kscratch = c.take<float>((size_t)w.nslots * 2 * (size_t)(n + 1));
+    w.pscratch = routes ? c.take<uint16_t>((size_t)w.nslots * K * (size_t)n) : nullptr;
+  }
   w.dscratch = (routes && !plain && n > 0) ? c.take<uint16_t>(fleet_dscratch_elems(n, K, w.cfg))
                                           : nullptr;
   w.bytes = c.off;
@@ -889,7 +891,8 @@ int sdp_split_fleet_eval(const sdp_split_args* a, int32_t max_routes, int32_t* n
       prof_end(st);
       if (e) return cuda_fail((cudaError_t)e, "split_fleet launch");
       // the flagged scenarios, if any
-      e = fleet_rescue_supported(a->n) ? launch_split_fleet_rescue(f, st) : launch_split_fleet_plain(f, st);
+      if (!w.cfg.band)
+        e = fleet_rescue_supported(a->n) ? launch_split_fleet_rescue(f, st) : launch_split_fleet_plain(f, st);
       if (e) return cuda_fail((cudaError_t)e, "split_fleet recompute launch");
     }
   }

@@ -312,6 +312,7 @@ size_t pipe_ring_bytes(int n_max, int Q, int64_t S, int B, bool batched);
 int launch_split_pipe(const PipeArgs& a, cudaStream_t st);
 
 // Fleet-limited Split (at most K routes, K <= 64): one warp per scenario
+// over the band of positions a split into K routes can use, or (long tours)
 // with the route-count layers across lanes, and a one-thread-per-scenario
 // layered kernel (PLAIN, and the recomputation of flagged scenarios).
 constexpr int kFleetMaxK = 64;
@@ -324,7 +325,7 @@ struct SplitFleetArgs {
   float* cost;               // [S]
   int32_t* nroutes;          // [S] or NULL
   uint8_t* route;            // [S*n] or NULL: route of each position, 0xFF if infeasible
-  uint16_t* dscratch;        // warp kernel with routes: fleet_dscratch_elems
+  uint16_t* dscratch;        // warp kernels with routes: fleet_dscratch_elems
   uint32_t* fb_list;         // warp kernel: flagged scenarios; plain: NULL = all S
   uint32_t* fb_count;
   float* kscratch;           // plain: [nslots * 2 * (n+1)]
@@ -335,6 +336,7 @@ struct SplitFleetArgs {
 struct FleetConfig {
   int warps;  // warps per CTA (0: the tour's records do not fit)
   int grid;
+  bool band;  // the band kernel, which also recomputes what it flags
 };
 FleetConfig fleet_config(int n, int K, int64_t S);
 size_t fleet_dscratch_elems(int n, int K, const FleetConfig& c);

@@ -11,7 +11,29 @@
 // psi_{k-1}(p) = K_{k-1}(p) + a_{p+1} -- the Split recursion fed by the layer
 // below -- and every layer has the same capacity window.
 //
-// split_fleet_kernel: one warp per scenario, the layers across its lanes:
+// split_fleet_band_kernel (AUTO up to n of about 1,700): one warp per
+// scenario, layer after layer, over the band of positions that matter.  A
+// split into at most K routes passes (k, i) only if n can be reached from i
+// with K - k more routes, i >= lo_k, and i from 0 with k, i <= hi_k: both
+// ends follow from the prefix loads alone (lo by filling routes greedily from
+// the tour's end, hi from its start), every feasible p of a position in the
+// band lies in the band below, so the values in it are those of the full
+// recursion.  A binding fleet leaves few routes of slack, and the band is
+// slack routes wide: at n = 500, Q = 200, K = 42 (about 41 needed) some 26
+// positions of 500.  Within a layer the positions are independent: a lane
+// each, windows by minima of blocks of B positions (built once per layer in
+// shared memory), values only.  The layers' psi rows go to a scratch of the
+// warp (band only, in L2), and the path is found from the last layer back,
+// 32 candidates at a time.
+//   Windows of at most 32 positions take blocks of 4; a scenario with a
+// longer one is flagged and recomputed by the same kernel with blocks of 16
+// (its list, SDP_FLAG_FALLBACK).
+//   n = 500, K = 42, S = 65,536: 1.12 ms where the deque kernel
+// below, which steps every layer through every position, took 5.43 ms and
+// 0.32 ms of recomputation.
+//
+// split_fleet_kernel (longer tours): one warp per scenario, the layers across
+// its lanes:
 // lane l's slot j holds layer k = 32 j + l + 1 (two slots: K <= 64).  Every
 // lane walks the same positions i = 1..n in lockstep, so the demand of s_i
 // and the tour record are broadcast loads; layer k's input psi_{k-1}(i-1) =
@@ -28,10 +50,7 @@
 // split_fleet_rescue_kernel recomputes it, one warp per scenario and the same
 // FP32 operations as split_fleet_plain_kernel (one thread per scenario, every
 // feasible p of every layer: PLAIN, and the recomputation for n too long for
-// the rescue's shared memory).  Rings of 16 entries, with 24 warps per CTA,
-// overflow on some scenarios of the n = 500, K = 42 workload but run it in
-// 5.4 ms of kernel where 32 entries and 16 warps took 9.0 ms; the one-thread
-// recomputation of the overflowing scenarios alone took 39 ms.
+// the rescue's shared memory).
 #include <math_constants.h>
 
 #include <algorithm>
@@ -460,6 +479,261 @@ __global__ void __launch_bounds__(kFRescueWarps * 32) split_fleet_rescue_kernel(
   }
 }
 
+// -------------------------------------------------------------- the band
+constexpr int kBandMaxWarps = 24;
+constexpr int kBandMinWarps = 8;   // per SM: fewer hide too little latency
+constexpr int kBandWindow = 32;    // longest window of the narrow form
+constexpr int kBandNarrow = 4, kBandWide = 16;  // positions per block minimum
+
+// CTA: a_{p+1} and ce_i [n+1] floats each, columns [n]; per warp: prefix
+// loads, psi and block minima [n+1 .. +16] (each on 16 bytes), window starts [n+1] uint16, and
+// the layers' ends and route bounds [K+2] uint16 x 3.
+__host__ __device__ constexpr size_t band_head(int n) {
+  return ((size_t)(n + 1) * 8 + (size_t)n * 2 + 15) & ~(size_t)15;
+}
+__host__ __device__ constexpr size_t band_floats(int n) { return ((size_t)n + 1 + kBandWide + 3) & ~(size_t)3; }
+__host__ __device__ constexpr size_t band_per_warp(int n, int K) {
+  return (band_floats(n) * 12 + (size_t)(n + 1) * 2 + (size_t)(K + 2) * 6 + 15) & ~(size_t)15;
+}
+
+// B: positions per block minimum.  LIST: the flagged scenarios (fb_list);
+// otherwise all, flagging those with a window above kBandWindow.
+template <int B, bool LIST, bool ROUTES>
+__global__ void __launch_bounds__(kBandMaxWarps * 32) split_fleet_band_kernel(SplitFleetArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int n = a.n, Q = a.Q, K = a.K;
+  float* as = reinterpret_cast<float*>(smem);  // a_{p+1} at [p], 0 at [n]
+  float* ces = as + n + 1;                     // ce_i at [i]
+  uint16_t* cols = reinterpret_cast<uint16_t*>(ces + n + 1);
+  unsigned char* wb = smem + band_head(n) + band_per_warp(n, K) * warp;
+  int32_t* L = reinterpret_cast<int32_t*>(wb);
+  float* psi = reinterpret_cast<float*>(L + band_floats(n));
+  float* blk = psi + band_floats(n);
+  uint16_t* pm = reinterpret_cast<uint16_t*>(blk + band_floats(n));
+  uint16_t* lo_of = pm + n + 1;      // [m]: the first position that m more routes take to n
+  uint16_t* hi_of = lo_of + K + 2;   // [k]: the last position that k routes reach
+  uint16_t* bound = hi_of + K + 2;   // route k covers positions bound[k] + 1 .. bound[k+1]
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const StepRec r = a.rec[k];
+    as[k] = r.a;
+    ces[k + 1] = r.ce;
+    cols[k] = (uint16_t)r.col;
+  }
+  if (threadIdx.x == 0) as[n] = 0.f;
+  __syncthreads();
+  const double Dn = *a.Dn;
+  const int64_t slot = (int64_t)blockIdx.x * nw + warp;
+  float* rows = ROUTES ? reinterpret_cast<float*>(a.dscratch) + slot * K * (int64_t)(n + 1) : nullptr;
+  bool neg = false;
+  uint32_t any_fb = 0, any_inf = 0;
+  const int64_t count = LIST ? (int64_t)*a.fb_count : a.S;
+  const int64_t stride = (int64_t)gridDim.x * nw;
+  const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(a.demands) & 15) == 0;
+  for (int64_t it = slot; it < count; it += stride) {
+    const int64_t s = LIST ? (int64_t)a.fb_list[it] : it;
+    const int32_t* qrow = a.demands + s * n;
+    if (!LIST && it + stride < count) {  // the next scenario's row into L2
+      const char* nx = reinterpret_cast<const char*>(a.demands + (s + stride) * n);
+      for (int o = lane * 128; o < n * 4; o += 32 * 128)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(nx + o));
+    }
+    // ---- demands by customer (staged in psi), then prefix loads in tour order
+    int32_t* stage = reinterpret_cast<int32_t*>(psi);
+    if (vec) {
+      for (int k = lane; k < n / 4; k += 32)
+        reinterpret_cast<int4*>(blk)[k] = __ldg(reinterpret_cast<const int4*>(qrow) + k);
+      stage = reinterpret_cast<int32_t*>(blk);
+    } else {
+      for (int k = lane; k < n; k += 32) stage[k] = __ldg(qrow + k);
+    }
+    __syncwarp();
+    bool over = false;
+    int carry = 0;
+    if (lane == 0) L[0] = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + lane;
+      int v = i < n ? stage[cols[i]] : 0;
+      neg |= v < 0;
+      over |= v > Q;
+      v = min(max(v, 0), Q + 1);
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(kAll, v, d);
+        if (lane >= d) v += t;
+      }
+      if (i < n) L[i + 1] = carry + v;
+      carry += __shfl_sync(kAll, v, 31);
+    }
+    bool infeasible = __any_sync(kAll, over);
+    __syncwarp();
+    float best = CUDART_INF_F;
+    int bk = 0;
+    if (!infeasible) {
+      // ---- window starts: the smallest p with L(i) - L(p) <= Q.  They only
+      // grow with i, so a lane's search begins at its last one's.
+      int lo = 0, longest = 0;
+      for (int i0 = 1; i0 <= n; i0 += 32) {
+        const int i = min(i0 + lane, n);
+        const int need = L[i] - Q;
+        int hi = i;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (L[mid] >= need) hi = mid; else lo = mid + 1;
+        }
+        pm[i] = (uint16_t)lo;
+        longest = max(longest, i - lo);
+      }
+      if (lane == 0) pm[0] = 0;
+      __syncwarp();
+      if (!LIST && __any_sync(kAll, longest > kBandWindow)) {
+        if (lane == 0) a.fb_list[atomicAdd(a.fb_count, 1u)] = (uint32_t)s;
+        any_fb = 1;
+        continue;
+      }
+      // ---- the band's lower end, from the tour's end
+      {
+        int x = n, m = 0;
+        for (; m <= K && x > 0; ++m) {
+          if (lane == 0) lo_of[m] = (uint16_t)x;
+          x = pm[x];
+        }
+        infeasible = x > 0;  // more than K routes (x reached 0 after m of them)
+        for (int k = m + lane; k <= K; k += 32) lo_of[k] = 0;
+      }
+      infeasible = infeasible || (__syncwarp(), lo_of[K] != 0);
+    }
+    if (!infeasible) {
+      // ---- layer 0
+      for (int p = lane; p < (int)band_floats(n); p += 32) {
+        psi[p] = p == 0 ? as[0] : CUDART_INF_F;
+        blk[p] = CUDART_INF_F;
+      }
+      if (lane == 0) hi_of[0] = 0;
+      __syncwarp();
+      int hi = 0, lo_prev = 0;
+      for (int k = 1; k <= K; ++k) {
+        // block minima of the layer below: blk[p] = min psi[p .. p + B - 1]
+        for (int p = lo_prev + lane; p <= hi; p += 32) {
+          float m = psi[p];
+#pragma unroll
+          for (int e = 1; e < B; ++e) m = fminf(m, psi[p + e]);
+          blk[p] = m;
+        }
+        // the last position that k routes reach
+        int nh = hi;
+        {
+          const int reach = L[hi] + Q;
+          for (;;) {
+            const int i = nh + 1 + lane;
+            const unsigned ok = __ballot_sync(kAll, i <= n && L[min(i, n)] <= reach);
+            nh += __popc(ok);
+            if (ok != kAll) break;
+          }
+        }
+        const int lo = max((int)lo_of[K - k], 1);
+        __syncwarp();
+        float* row = ROUTES ? rows + (int64_t)(k - 1) * (n + 1) : nullptr;
+        for (int top = nh; top >= lo; top -= 32) {
+          const int i = max(top - lane, lo);
+          const int pi = pm[i];
+          float m = CUDART_INF_F;
+          const int last = i - B;  // the block that ends at i - 1
+          if (last >= pi) {
+            m = blk[last];
+            for (int p = pi; p < last; p += B) m = fminf(m, blk[p]);
+          } else {
+            for (int p = pi; p < i; ++p) m = fminf(m, psi[p]);
+          }
+          const float Ki = __fadd_rn(m, ces[i]);
+          __syncwarp();  // this round's reads come before its writes
+          if (top - lane >= lo) {
+            const float v = __fadd_rn(Ki, as[i]);
+            psi[i] = v;
+            if (ROUTES) row[i] = v;
+          }
+          if (top == n) {
+            const float Kn = __shfl_sync(kAll, Ki, 0);
+            if (Kn < best) {  // the fewest routes on ties
+              best = Kn;
+              bk = k;
+            }
+          }
+        }
+        if (k == 1 && lane == 0) psi[0] = CUDART_INF_F;  // J_k(0), k >= 1
+        if (lane == 0) hi_of[k] = (uint16_t)nh;
+        hi = nh;
+        lo_prev = lo_of[K - k];
+        __syncwarp();
+      }
+      infeasible = bk == 0;
+    }
+    any_inf |= infeasible;
+    if (lane == 0) {
+      a.cost[s] = infeasible ? CUDART_INF_F : (float)((double)best + Dn);
+      if (a.nroutes) a.nroutes[s] = infeasible ? 0 : bk;
+    }
+    if (ROUTES) {
+      uint8_t* out = a.route + s * n;
+      uint8_t* st = reinterpret_cast<uint8_t*>(psi);
+      if (infeasible) {
+        for (int m = lane; m < n; m += 32) out[m] = 0xFFu;
+      } else {
+        // ---- the path, last route first: the smallest p of the window with
+        // the least psi of the layer below
+        int i = n;
+        for (int k = bk; k >= 1; --k) {
+          if (lane == 0) bound[k] = (uint16_t)i;
+          int p = 0;
+          if (k > 1) {
+            const float* row = rows + (int64_t)(k - 2) * (n + 1);
+            const int p0 = max((int)pm[i], 1), p1 = min(i - 1, (int)hi_of[k - 1]);
+            p = p0;
+            uint32_t least = 0xFFFFFFFFu;
+            for (int c = p0; c <= p1; c += 32) {
+              // floats as unsigned keys in their order (-0 taken as 0)
+              uint32_t key = 0xFFFFFFFFu;
+              if (c + lane <= p1) {
+                const uint32_t b = __float_as_uint(__fadd_rn(row[c + lane], 0.f));
+                key = b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+              }
+              const uint32_t m = __reduce_min_sync(kAll, key);
+              if (m < least) {
+                least = m;
+                p = c + __ffs(__ballot_sync(kAll, key == m)) - 1;
+              }
+            }
+          }
+          i = p;
+        }
+        if (lane == 0) bound[0] = 0;
+        __syncwarp();
+        if (LIST) {
+          for (int k = 0; k < bk; ++k)
+            for (int m = bound[k] + lane; m < (int)bound[k + 1]; m += 32) st[m] = (uint8_t)k;
+        } else {
+          for (int k = lane; k < bk; k += 32)
+            for (int m = bound[k]; m < (int)bound[k + 1]; ++m) st[m] = (uint8_t)k;
+        }
+        __syncwarp();
+        if ((n & 3) == 0 && (reinterpret_cast<uintptr_t>(a.route) & 3) == 0) {
+          for (int m = lane; m < n / 4; m += 32)
+            reinterpret_cast<uint32_t*>(out)[m] = reinterpret_cast<const uint32_t*>(st)[m];
+        } else {
+          for (int m = lane; m < n; m += 32) out[m] = st[m];
+        }
+      }
+    }
+    __syncwarp();  // the scenario's shared rows are read before the next one's writes
+  }
+  if (lane == 0) {
+    if (any_fb) atomicOr(a.status, SDP_FLAG_FALLBACK);
+    if (any_inf) atomicOr(a.status, SDP_FLAG_INFEASIBLE);
+  }
+  if (__any_sync(kAll, neg) && lane == 0) atomicOr(a.status, SDP_FLAG_NEG_INPUT);
+}
+
 size_t fleet_head(int n) { return (((size_t)n * 8 + (size_t)n * 2) + 255) & ~(size_t)255; }
 size_t fleet_per_warp(int ks) { return (size_t)ks * kFRingBytes + 256 * 4; }
 
@@ -473,11 +747,37 @@ int launch_fleet_k(const SplitFleetArgs& a, int warps, int grid, cudaStream_t st
   return (int)cudaGetLastError();
 }
 
+template <bool ROUTES>
+int launch_band(const SplitFleetArgs& a, const FleetConfig& c, cudaStream_t st) {
+  const size_t smem = band_head(a.n) + band_per_warp(a.n, a.K) * c.warps;
+  auto narrow = split_fleet_band_kernel<kBandNarrow, false, ROUTES>;
+  auto wide = split_fleet_band_kernel<kBandWide, true, ROUTES>;
+  cudaError_t e = cudaFuncSetAttribute(narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return (int)e;
+  narrow<<<c.grid, c.warps * 32, smem, st>>>(a);
+  wide<<<c.grid, c.warps * 32, smem, st>>>(a);
+  return (int)cudaGetLastError();
+}
+
 }  // namespace
 
 // One CTA per SM with as many warps as its shared memory holds (up to 16);
 // fewer CTAs when there are fewer scenarios.
 FleetConfig fleet_config(int n, int K, int64_t S) {
+  if (band_head(n) + band_per_warp(n, K) * kBandMinWarps <= 226 * 1024) {
+    int warps = (int)((226 * 1024 - band_head(n)) / band_per_warp(n, K));
+    warps = warps > kBandMaxWarps ? kBandMaxWarps : warps;
+    // few scenarios: as many SMs as possible
+    const int64_t share = (S + num_sms() - 1) / num_sms();
+    FleetConfig c{};
+    c.band = true;
+    c.warps = (int)imin64(warps, share < 1 ? 1 : share);
+    const int64_t need = (S + c.warps - 1) / c.warps;
+    c.grid = (int)imin64(need < 1 ? 1 : need, (int64_t)num_sms());
+    return c;
+  }
   const int ks = K <= 32 ? 1 : 2;
   const size_t budget = 226 * 1024;  // dynamic shared memory of one CTA per SM
   const size_t head = fleet_head(n);
@@ -492,12 +792,14 @@ FleetConfig fleet_config(int n, int K, int64_t S) {
 }
 
 size_t fleet_dscratch_elems(int n, int K, const FleetConfig& c) {
+  if (c.band) return (size_t)c.grid * c.warps * (size_t)K * (size_t)(n + 1) * 2;  // floats
   const int ks = K <= 32 ? 1 : 2;
   return (size_t)c.grid * c.warps * (size_t)n * 32 * ks;
 }
 
 int launch_split_fleet(const SplitFleetArgs& a, const FleetConfig& c, cudaStream_t st) {
   if (c.warps < 1) return (int)cudaErrorInvalidValue;
+  if (c.band) return a.route ? launch_band<true>(a, c, st) : launch_band<false>(a, c, st);
   if (a.K <= 32)
     return a.route ? launch_fleet_k<1, true>(a, c.warps, c.grid, st)
                    : launch_fleet_k<1, false>(a, c.warps, c.grid, st);
