@@ -461,9 +461,9 @@ int check_ws(void* ws, size_t have, size_t need) {
 }
 
 // Runs the chosen DP kernel over all S, then recomputes the scenarios it
-// flagged (one warp each where split_rescue.cu applies: hard capacity, no
-// route histogram; else the plain kernel over the flagged list), or runs the
-// PLAIN kernel over all S.
+// flagged (one warp each where its rows fit split_rescue.cu's shared memory;
+// else the plain kernel over the flagged list), or runs the PLAIN kernel over
+// all S.
 int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
                    unsigned long long* hist, cudaStream_t st) {
   int algo = resolve_algo(a);
@@ -554,11 +554,12 @@ int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
     prof_end(st);
     if (e) return cuda_fail((cudaError_t)e, "split_deque launch");
   }
-  if (algo != SDP_ALGO_PLAIN && !hist && a->capacity_mode != SDP_CAPACITY_SOFT &&
-      rescue_supported(a->n)) {
+  const bool soft = a->capacity_mode == SDP_CAPACITY_SOFT;
+  if (algo != SDP_ALGO_PLAIN && rescue_supported(a->n, soft, hist != nullptr)) {
     // the scenarios the DP kernel flagged, one warp each
     RescueArgs r{};
     r.batched = 0; r.Q = a->Q; r.S = a->S; r.n_max = a->n; r.n1 = a->n;
+    r.soft = soft ? 1 : 0; r.beta = a->overload_penalty; r.hist = hist;
     r.fb_list1 = w.fb_list; r.cost = cost; r.pred = pred; r.pred_dtype = a->pred_dtype;
     r.rec = w.prep.rec; r.Dn = w.prep.Dn; r.demands = a->demands;
     r.fb_count = w.fb_count; r.status = status;

@@ -172,14 +172,17 @@ struct BatchFallbackArgs {
 };
 void launch_batch_fallback(const BatchFallbackArgs& a, cudaStream_t st);
 
-// Warp-per-scenario recomputation of flagged hard-capacity scenarios
-// (split_rescue.cu), one tour or a batched plan's entries; the same FP32
-// results as the plain kernel.
+// Warp-per-scenario recomputation of flagged scenarios (split_rescue.cu), one
+// tour (hard or soft capacity, or its route counts) or a batched plan's
+// entries; the same FP32 results as the plain kernel.
 struct RescueArgs {
   int batched;
   int Q;
   int64_t S;
-  int n_max;                   // longest tour (shared memory per warp: 8 (n_max+1) bytes)
+  int n_max;                   // longest tour (shared memory per warp: 8..12 (n_max+1) bytes)
+  int soft;                    // one tour: soft capacity, beta per unit of route load above Q
+  float beta;
+  unsigned long long* hist;    // one tour, hard: route counts [2n+1] instead of costs, or NULL
   // one tour
   int n1;
   const uint32_t* fb_list1;    // [*fb_count] scenario ids
@@ -199,7 +202,7 @@ struct RescueArgs {
   const uint32_t* fb_count;
   uint32_t* status;
 };
-bool rescue_supported(int n_max);
+bool rescue_supported(int n_max, bool soft, bool hist);
 // max_work: the most entries the list can hold (sizes the grid)
 int launch_split_rescue(const RescueArgs& a, int64_t max_work, cudaStream_t st);
 int launch_split_batch(const BatchKernelArgs& a, int warps, int ring, int ns, int grid,

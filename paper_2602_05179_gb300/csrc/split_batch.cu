@@ -175,7 +175,7 @@ int enqueue(sdp_plan* p, cudaStream_t st, uint32_t* status, bool with_events) {
   }
   if (with_events) cudaEventRecordWithFlags(p->ev1, st, cudaEventRecordExternal);
   if (e) return pcuda((cudaError_t)e, "batch kernel");
-  if (rescue_supported(p->n_max)) {
+  if (rescue_supported(p->n_max, false, false)) {
     // the entries the DP kernel flagged, one warp each
     RescueArgs r{};
     r.batched = 1; r.Q = p->Q; r.S = p->S; r.n_max = p->n_max;

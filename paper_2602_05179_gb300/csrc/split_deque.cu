@@ -1294,7 +1294,7 @@ __global__ void __launch_bounds__(MAXT, 1) split_tmem_adj_kernel(SplitDequeArgs 
 // Soft-capacity Split with TMEM staging (16 warps per SM, as split_tmem_kernel
 // with XW = 0): every split is allowed and a route pays beta per unit of
 // load above Q.  Demands are staged exactly (no clamp to Q + 1); a row with a
-// demand the staging type cannot hold goes to the plain kernel.
+// demand the staging type cannot hold is recomputed (split_rescue.cu).
 template <typename QT, typename PT, int OUT>
 __global__ void __launch_bounds__(512, 1) split_tmem_soft_kernel(SplitDequeArgs a, int64_t tiles) {
   constexpr int RING = 16;

@@ -818,7 +818,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_pipe_kernel(PipeArgs a) {
             // [0, Q+1] (the tile takes the checked step, the scenario is
             // infeasible).  Soft: kept exactly for the checked step up to
             // kSoftMax (so that Q + q < 2^16 in the front test); beyond it
-            // the scenario goes to the plain kernel.
+            // the scenario is recomputed (split_rescue.cu).
             bool inf = false, big = false;
             word = 0u;
 #pragma unroll
