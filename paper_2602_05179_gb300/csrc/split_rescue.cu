@@ -13,7 +13,7 @@
 // and half a dozen operations on the dependent chain, where spreading its
 // candidates over the lanes and reducing them cost a chain of ten shuffles
 // and several loads: 112 us for the flagged scenarios of an n = 333 call with
-// that form, @@H@@ us with this one.
+// that form, 25 us with this one.
 //   Soft capacity lets every earlier p compete.  A lane scans them downward
 // and stops where even the least psi so far (PM, a running minimum) with the
 // penalty reached exceeds its best: penalties only grow as p falls and
