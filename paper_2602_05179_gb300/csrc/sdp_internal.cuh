@@ -314,6 +314,12 @@ int pipe_grid(int64_t S, int B, bool batched);
 size_t pipe_ring_bytes(int n_max, int Q, int64_t S, int B, bool batched);
 int launch_split_pipe(const PipeArgs& a, cudaStream_t st);
 
+// Batched plans whose tours have one length and share one demand array
+// (split_shared.cu): the batched arguments of the pipelined kernel (order,
+// qt, counter and stride unused; n_max the tours' length).
+bool shared_supported(int n, int Q, int B);
+int launch_split_shared(const PipeArgs& a, cudaStream_t st);
+
 // Fleet-limited Split (at most K routes, K <= 64): one warp per scenario
 // over the band of positions a split into K routes can use, or (long tours)
 // with the route-count layers across lanes, and a one-thread-per-scenario

@@ -9,7 +9,9 @@
 // kernel over (tour, 32-scenario tile) items -> recomputation of the
 // scenarios it flagged (one warp each, split_rescue.cu, where the longest
 // tour fits its shared memory; else the plain per-scenario kernel) ->
-// per-tour FP64 means], captured once in a CUDA graph and replayed.  The persistent kernel is the pipelined one
+// per-tour FP64 means], captured once in a CUDA graph and replayed.  The
+// persistent kernel is split_shared.cu's where at least 64 tours of one length
+// share one demand array (the SAA search); else the pipelined one
 // (split_pipe_kernel: producer warps narrow each tile's rows into tour order
 // in an L2-resident slot ring, 23 DP warps per SM) when the demand offsets
 // allow bulk copies and every tour has n <= 1024, else the streaming one
@@ -48,6 +50,7 @@ struct sdp_plan {
   unsigned long long* d_total = nullptr;
   unsigned char* d_qt = nullptr;  // row slots of the streaming kernel, or NULL
   unsigned char* d_pq = nullptr;  // slot ring of the pipelined kernel, or NULL
+  bool shared = false;            // one length and one demand array for every tour
   // caller's arrays
   const int32_t* tours = nullptr;
   const float* coords = nullptr;
@@ -161,7 +164,7 @@ int enqueue(sdp_plan* p, cudaStream_t st, uint32_t* status, bool with_events) {
     pa.qt = p->d_pq; pa.stride = pipe_row_stride(p->n_max, p->Q); pa.counter = p->d_counter;
     pa.n_max = p->n_max;
     pa.fb_count = p->d_fb_count; pa.fb_list = p->d_fb_list; pa.status = status;
-    e = launch_split_pipe(pa, st);
+    e = p->shared ? launch_split_shared(pa, st) : launch_split_pipe(pa, st);
   } else if (p->warps < 0) {
     BatchStreamArgs sa{};
     sa.B = p->B; sa.Q = p->Q; sa.S = p->S;
@@ -299,6 +302,10 @@ int sdp_split_plan_create(const sdp_split_batch_desc* d, sdp_plan** out) {
   if (stream_ok && pipe_supported(p->n_max, p->Q))
     chk(alloc_copy<unsigned char>(&p->d_pq, nullptr,
                                   pipe_ring_bytes(p->n_max, p->Q, p->S, p->B, true)));
+  // tours of one length on one demand array: a tile staged once for all of them
+  p->shared = p->d_pq != nullptr && shared_supported(p->n_max, p->Q, p->B);
+  for (int b = 1; p->shared && b < d->B; ++b)
+    p->shared = d->n_host[b] == d->n_host[0] && d->dem_off_host[b] == d->dem_off_host[0];
   if (e == cudaSuccess) e = cudaEventCreate(&p->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&p->ev1);
   if (e != cudaSuccess) {
