@@ -289,6 +289,7 @@ struct PipeArgs {
   int pred_dtype;
   unsigned char* qt;           // slot ring, pipe_ring_bytes
   int nslot;                   // slots per CTA (set by launch_split_pipe)
+  uint32_t item_cap;           // one tour: tiles a CTA takes at most, 0: no limit (set by launch_split_pipe)
   int n_max;                   // batched: the longest tour
   int soft;                    // one tour: soft capacity, beta per unit of route load above Q
   float beta;

@@ -112,6 +112,13 @@ constexpr uint32_t kOutBytes = 32u * 32u;      // predecessor stage per warp: 32
 constexpr int kColsStride = kPipeMaxN + 8;     // uint16 entries per column table
 template <typename QT>
 __host__ __device__ constexpr int soft_max() { return sizeof(QT) == 1 ? 255 : 32767; }
+// The first items of a CTA are narrowed four rows at a time: n = 500 then gets a
+// tile every 2.6 us instead of 3.9 (n = 1000, 16-bit: 6.5 instead of 10.2), which
+// is what a launch of at most a tile per DP warp waits for (n = 1000, Q = 400,
+// S = 10^5: 0.349 -> 0.28 ms).  Once the DP warps are busy the faster narrowing
+// only takes their issue slots (n = 500, S = 10^6: +1%; the 1,024-tour plan +3%).
+constexpr int kCapRounds = 5;  // launches of up to so many tiles per DP warp share them evenly
+constexpr uint32_t kRampItems = (uint32_t)kDp + 5u;
 constexpr int kCheckEvery = 2;                 // steps between ring tests (lean step)
 constexpr uint32_t kMaxAtCheck = 14u;          // entries allowed at a test (+2 pushes <= 16)
 static_assert(kMaxAtCheck + kCheckEvery <= (uint32_t)kRing && 16 % kCheckEvery == 0,
@@ -373,12 +380,23 @@ struct SmemRec2 {
     asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(base + 8u * (uint32_t)k));
     return v;
   }
+  // positions k + 1 and k + 2, k even: one load for two steps
+  __device__ __forceinline__ float4 pair(int k) const {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(base + 8u * (uint32_t)k));
+    return v;
+  }
 };
 struct GlobalRec2 {
   const StepRec* p;
   __device__ __forceinline__ float2 operator()(int k) const {
     const float4 v = __ldg(reinterpret_cast<const float4*>(p + k));
     return make_float2(v.y, v.z);
+  }
+  __device__ __forceinline__ float4 pair(int k) const {
+    const float2 v = (*this)(k), w = (*this)(k + 1);
+    return make_float4(v.x, v.y, w.x, w.y);
   }
 };
 
@@ -498,10 +516,13 @@ __device__ __forceinline__ void pipe_tile(int n, int Q, float beta, const unsign
     uint4 nx[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) nx[v] = ld_cg_v4(src + V * bn + v);
+    constexpr bool kPairs = !(PRED && sizeof(PT) == 2);
+    float4 rp;
 #pragma unroll
     for (int u = 0; u < E; ++u) {
       const int i = b * E + u + 1;
-      const float2 r = rec(i - 1);
+      if (kPairs && (u & 1) == 0) rp = rec.pair(i - 1);
+      const float2 r = !kPairs ? rec(i - 1) : (u & 1) ? make_float2(rp.z, rp.w) : make_float2(rp.x, rp.y);
       const uint32_t qh = q_at<QT>(c, u);
       do_step(i, qh, r, u % kCheckEvery == kCheckEvery - 1);
       if (PRED) {
@@ -530,7 +551,8 @@ __device__ __forceinline__ void pipe_tile(int n, int Q, float beta, const unsign
 }
 
 // ------------------------------------------------------------------ kernel
-template <typename QT, typename PT, bool PRED, bool BATCH, bool SOFT, int NST>
+// RAMP: a launch of few rounds (see kCapRounds)
+template <typename QT, typename PT, bool PRED, bool BATCH, bool SOFT, int NST, bool RAMP>
 __global__ void __launch_bounds__(kThreads, 1) split_pipe_kernel(PipeArgs a) {
   constexpr int kNStage = NST;  // producer stages of this launch
   static_assert(NST >= 2 && NST <= kMaxNStage, "stage count");
@@ -612,7 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_pipe_kernel(PipeArgs a) {
     auto wait_done = [&](int64_t y) -> bool {
       return y < 0 || mbar_wait_abortable(empty_of(y), par_of(y), &abort_flag, a.wait_ns);
     };
-    while (!failed) {
+    while (!failed && (!RAMP || li < a.item_cap)) {
       int64_t gid = 0;
       if (lane == 0) gid = (int64_t)atomicAdd(a.counter, 1ull);
       gid = __shfl_sync(0xffffffffu, gid, 0);
@@ -791,11 +813,49 @@ __global__ void __launch_bounds__(kThreads, 1) split_pipe_kernel(PipeArgs a) {
       const int rows = mt.rows;
       const uint32_t sq_b = smem_u32(smem) + (uint32_t)st * kStage;
       uint32_t* out = reinterpret_cast<uint32_t*>(qslots + ((int64_t)slot * 32 + mt.rbase) * a.stride);
+      // Four rows at a time, their loads in flight together, while the DP warps
+      // wait for their first tiles (kRampItems); what is left of the rows, or
+      // all of them where a demand is above Q or below 0, goes to the loop below.
+      int rbeg = rfirst;
+      if (RAMP && mt.item < kRampItems) {
+        uint32_t mx = 0u;
+        const uint32_t rpitch = 4u * (uint32_t)rstep * (uint32_t)n;
+        const int opitch = rstep * sw;
+        const int fours = rows > rfirst ? ((rows - rfirst + rstep - 1) / rstep) / 4 : 0;
+#pragma unroll
+        for (int j = 0; j < kWords; ++j) {
+          const int k = kw0 + kHalf * j;
+          if (k < wq) {
+            uint32_t rb = sq_b + (uint32_t)(rfirst * n) * 4u;
+            uint32_t* o = out + (int64_t)rfirst * sw + k;
+#pragma unroll 1
+            for (int it = 0; it < fours; ++it, rb += 4u * rpitch, o += 4 * opitch) {
+              int v[4][PER];
+#pragma unroll
+              for (int g = 0; g < 4; ++g)
+#pragma unroll
+                for (int e = 0; e < PER; ++e)
+                  asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v[g][e]) : "r"(rb + (uint32_t)g * rpitch + wcol[j][e]));
+#pragma unroll
+              for (int g = 0; g < 4; ++g) {
+#pragma unroll
+                for (int e = 0; e < PER; ++e) mx = max(mx, (uint32_t)v[g][e]);
+                const uint32_t word = sizeof(QT) == 1
+                                          ? __byte_perm(__byte_perm(v[g][0], v[g][1 % PER], 0x0040),
+                                                        __byte_perm(v[g][2 % PER], v[g][3 % PER], 0x0040), 0x5410)
+                                          : __byte_perm(v[g][0], v[g][1 % PER], 0x5410);
+                o[g * opitch] = word & wmask[j];
+              }
+            }
+          }
+        }
+        if (mx <= (uint32_t)Q) rbeg += 4 * fours * rstep;
+      }
 #pragma unroll
       for (int j = 0; j < kWords; ++j) {
         const int k = kw0 + kHalf * j;
         if (k >= wq) break;
-        const int r0 = rfirst;
+        const int r0 = rbeg;
         uint32_t rb = sq_b + (uint32_t)(r0 * n) * 4u;  // stage row r0
         uint32_t* o = out + (int64_t)r0 * sw + k;
         int r = r0;
@@ -952,14 +1012,20 @@ size_t pipe_smem(const PipeArgs& a, bool pred) {
          (a.batched ? 2 * (size_t)kColsStride : (size_t)n + 8) * sizeof(uint16_t);
 }
 
-template <typename QT, typename PT, bool PRED, bool BATCH, bool SOFT = false, int NST = 2>
-int launch_k(const PipeArgs& a, cudaStream_t st) {
-  auto k = split_pipe_kernel<QT, PT, PRED, BATCH, SOFT, NST>;
+template <typename QT, typename PT, bool PRED, bool BATCH, bool SOFT, int NST, bool RAMP>
+int launch_r(const PipeArgs& a, cudaStream_t st) {
+  auto k = split_pipe_kernel<QT, PT, PRED, BATCH, SOFT, NST, RAMP>;
   const size_t smem = pipe_smem(a, PRED);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
   k<<<pipe_grid(a.S, a.B, BATCH), kThreads, smem, st>>>(a);
   return (int)cudaGetLastError();
+}
+template <typename QT, typename PT, bool PRED, bool BATCH, bool SOFT = false, int NST = 2>
+int launch_k(const PipeArgs& a, cudaStream_t st) {
+  if constexpr (!BATCH)
+    if (a.item_cap > 0u) return launch_r<QT, PT, PRED, BATCH, SOFT, NST, true>(a, st);
+  return launch_r<QT, PT, PRED, BATCH, SOFT, NST, false>(a, st);
 }
 
 template <typename QT>
@@ -1005,6 +1071,17 @@ int launch_split_pipe(const PipeArgs& a0, cudaStream_t st) {
   PipeArgs a = a0;
   if (a.wait_ns == 0) a.wait_ns = kWaitLimitNs;
   a.nslot = pipe_slots(a.S, a.B, a.batched != 0);
+  // One tour of at most kCapRounds tiles per DP warp: no CTA claims more than
+  // its even share.  The issuers claim up to kSlots tiles ahead of their DP
+  // warps, so the first CTAs to run took tiles that others had idle warps for
+  // (n = 500, no predecessors, 23 tiles per CTA: 182 -> 160 us; 46: 305 -> 270).
+  // Launches of more rounds even out by themselves, and keep the kernel
+  // without the ramp's code (1% at n = 500, S = 10^6).
+  a.item_cap = 0u;
+  if (!a.batched) {
+    const int64_t grid = pipe_grid(a.S, 1, false), tiles = (a.S + 31) / 32;
+    if (tiles <= grid * kDp * kCapRounds) a.item_cap = (uint32_t)((tiles + grid - 1) / grid);
+  }
   return a.Q <= 254 ? launch_q<uint8_t>(a, st) : launch_q<uint16_t>(a, st);
 }
 
