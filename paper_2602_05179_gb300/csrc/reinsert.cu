@@ -41,6 +41,7 @@ __host__ __device__ constexpr int bits_stride(int kc) { return (kc + 7) & ~7; }
 template <int KC, bool TABLE, bool UNIT>
 __global__ void __launch_bounds__(512) reinsert_kernel(ReinsertArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  if (a.mean_counter && blockIdx.x == 0 && threadIdx.x == 0) *a.mean_counter = 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int T = a.T, U = a.U;
   constexpr int GW = kPad + 32 * KC;
@@ -201,6 +202,7 @@ constexpr int kUnrolledRoutes = 8;
 template <int KC, bool UNIT>
 __global__ void __launch_bounds__(512) reinsert_routes_kernel(ReinsertArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  if (a.mean_counter && blockIdx.x == 0 && threadIdx.x == 0) *a.mean_counter = 0u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int T = a.T, U = a.U, K = a.n_routes;
   constexpr int GW = kPad + 32 * KC;
@@ -425,6 +427,7 @@ struct IntTag {
 template <int KC, bool TABLE, bool UNIT, int RK = 0>
 __global__ void __launch_bounds__(kLaneWarps * 32, 1) reinsert_lane_kernel(ReinsertArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  if (a.mean_counter && blockIdx.x == 0 && threadIdx.x == 0) *a.mean_counter = 0u;
   constexpr int NI = 32 * KC;  // rows
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int T = a.T, U = a.U;

@@ -217,7 +217,7 @@ struct SplitWs {
   unsigned long long* hist;
   unsigned char* qt;   // STREAM: narrowed demands in tour order
   uint32_t* tflags;    // STREAM: per-tile rows with a demand above Q
-  unsigned long long* counter;  // PIPE: group queue (zeroed before each launch)
+  unsigned long long* counter;  // PIPE: group queue (zeroed with fb_count)
   uint32_t* dscratch;  // fused adjoint on TMEM: i - pred(i) per [word][lane]
   size_t bytes;
 };
@@ -283,7 +283,9 @@ SplitWs carve_split(const sdp_split_args* a, void* base, bool backward) {
   w.prep.cols = c.take<uint16_t>((size_t)n);
   w.prep.Dn = c.take<double>(1);
   w.mean_partial = c.take<double>(kMeanBlocks);
-  w.fb_count = c.take<uint32_t>(1);
+  // flagged scenarios, and the tiles claimed 8 bytes on
+  w.fb_count = c.take<uint32_t>(4);
+  w.counter = w.fb_count ? reinterpret_cast<unsigned long long*>(w.fb_count + 2) : nullptr;
   if (algo == SDP_ALGO_DEQUE || algo == SDP_ALGO_STREAM || algo == SDP_ALGO_PIPE) {
     w.fb_list = c.take<uint32_t>((size_t)a->S);
     w.nslots = a->S < kFallbackSlots ? a->S : kFallbackSlots;
@@ -300,13 +302,11 @@ SplitWs carve_split(const sdp_split_args* a, void* base, bool backward) {
                    : nullptr;
   w.qt = nullptr;
   w.tflags = nullptr;
-  w.counter = nullptr;
   if (algo == SDP_ALGO_PIPE && !backward && n > 0) {
     const int64_t rows = (n > 0 && is_host_ptr(a->demands))
                              ? (a->S < kHostChunkRows ? a->S : kHostChunkRows)
                              : a->S;
     w.qt = c.take<unsigned char>(pipe_ring_bytes(n, a->Q, rows, 1, false));
-    w.counter = c.take<unsigned long long>(1);
   }
   if (algo == SDP_ALGO_STREAM && !backward && n > 0) {
     const int64_t rows = (n > 0 && is_host_ptr(a->demands))
@@ -374,7 +374,7 @@ int run_split_host_chunks(const sdp_split_args* a, const SplitWs& w, uint32_t* s
                           cudaMemcpyHostToDevice, hp.copy);
     if (e == cudaSuccess) e = cudaEventRecord(hp.ready[b], hp.copy);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, hp.ready[b], 0);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.fb_count, 0, sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.fb_count, 0, 4 * sizeof(uint32_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "host pipeline copy");
     sdp_split_args c = *a;
     c.S = cnt;
@@ -501,8 +501,6 @@ int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
     const uint64_t stall = fault_stall_ns();
     pa.wait_ns = stall ? stall : kWaitLimitNs;
     pa.stall = stall ? 1 : 0;
-    cudaError_t ce = cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long), st);
-    if (ce != cudaSuccess) return cuda_fail(ce, "pipe counter reset");
     note_launch(32, pipe_grid(a->S, 1, false));  // 23 DP + 1 issuing + 8 narrowing warps
     prof_begin(st);
     const int e = launch_split_pipe(pa, st);
@@ -703,9 +701,11 @@ int sdp_split_eval(const sdp_split_args* args, void* stream) {
   const SplitWs w = carve_split(a, a->workspace, false);
   if (a->S > 0 && a->n == 0) {
     cudaError_t e = cudaMemsetAsync(a->cost_out, 0, sizeof(float) * a->S, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(mean_counter(w.mean_partial), 0, sizeof(uint32_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "memset cost");
   } else if (a->S > 0) {
-    launch_tour_prep(a->tour, a->n, a->coords, a->dist, w.prep, status, w.fb_count, st);
+    launch_tour_prep(a->tour, a->n, a->coords, a->dist, w.prep, status,
+                     {w.fb_count, w.counter, mean_counter(w.mean_partial)}, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "tour_prep launch");
     // host demands: copied chunk by chunk (from the caller's host address)
@@ -866,9 +866,11 @@ int sdp_split_fleet_eval(const sdp_split_args* a, int32_t max_routes, int32_t* n
   if (a->S > 0 && a->n == 0) {
     cudaError_t e = cudaMemsetAsync(a->cost_out, 0, sizeof(float) * a->S, st);
     if (e == cudaSuccess && nroutes_out) e = cudaMemsetAsync(nroutes_out, 0, sizeof(int32_t) * a->S, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(mean_counter(w.mean_partial), 0, sizeof(uint32_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "memset fleet outputs");
   } else if (a->S > 0) {
-    launch_tour_prep(a->tour, a->n, a->coords, a->dist, w.prep, status, w.fb_count, st);
+    launch_tour_prep(a->tour, a->n, a->coords, a->dist, w.prep, status,
+                     {w.fb_count, nullptr, mean_counter(w.mean_partial)}, st);
     SplitFleetArgs f{};
     f.n = a->n; f.Q = a->Q; f.K = max_routes; f.S = a->S;
     f.rec = w.prep.rec; f.Dn = w.prep.Dn; f.demands = a->demands;
@@ -933,7 +935,7 @@ int sdp_split_count_arcs(const sdp_split_args* args, int64_t* arcs_out, uint64_t
     }
     return SDP_OK;
   }
-  launch_tour_prep(a->tour, a->n, a->coords, a->dist, w.prep, status, w.fb_count, st);
+  launch_tour_prep(a->tour, a->n, a->coords, a->dist, w.prep, status, {w.fb_count, nullptr, nullptr}, st);
   launch_count_arcs(a->n, a->Q, a->S, w.prep.rec, a->demands, arcs_out,
                     reinterpret_cast<unsigned long long*>(total_out), 4 * num_sms(), st);
   cudaError_t e = cudaGetLastError();
@@ -974,14 +976,14 @@ int sdp_split_backward(const sdp_split_args* args, const void* pred, const float
     if (pred) {
       launch_backtrack_hist(n, fwd->S, pred, fwd->pred_dtype, w.hist, status, st);
     } else {
-      launch_tour_prep(fwd->tour, n, fwd->coords, fwd->dist, w.prep, status, w.fb_count, st);
+      launch_tour_prep(fwd->tour, n, fwd->coords, fwd->dist, w.prep, status,
+                       {w.fb_count, w.counter, nullptr}, st);
       rc = run_split_core(fwd, w, status, w.hist, st);
       if (rc) return rc;
     }
   }
-  launch_grad_assemble(n, fwd->S, fwd->tour, w.hist, grad_mean, grad_dist, route_hist_out, st);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "backward launch");
+  const int ge = launch_grad(n, fwd->S, fwd->tour, w.hist, grad_mean, false, grad_dist, route_hist_out, st);
+  if (ge) return cuda_fail((cudaError_t)ge, "backward launch");
   return SDP_OK;
 }
 
@@ -1064,6 +1066,7 @@ int sdp_reinsert_eval(const sdp_reinsert_args* a, void* stream) {
                              static_cast<unsigned char*>(a->workspace) +
                              align_up((size_t)kMeanBlocks * sizeof(double), 256))
                        : nullptr;
+  r.mean_counter = a->mean_out ? mean_counter(static_cast<double*>(a->workspace)) : nullptr;
   prof_begin(st);
   int e = launch_reinsert(r, st);
   prof_end(st);

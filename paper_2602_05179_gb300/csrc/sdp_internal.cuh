@@ -39,10 +39,17 @@ struct TourPrep {
 // ----------------------------------------------------------------- kernels
 // status bits are OR-ed into *status (a per-device __device__ word).
 
+// Counters of a call that its first kernel sets to zero (NULL: none): flagged
+// scenarios, tiles claimed, blocks of the mean done.
+struct CallCounters {
+  uint32_t* flagged;
+  unsigned long long* tiles;
+  uint32_t* mean;
+};
 // one CTA per tour; coords or dist mode
 void launch_tour_prep(const int32_t* tour, int n, const float* coords,
                       const float* dist, TourPrep prep, uint32_t* status,
-                      uint32_t* reset_word, cudaStream_t st);
+                      CallCounters counters, cudaStream_t st);
 
 struct SplitPlainArgs {
   int n, Q;
@@ -362,14 +369,19 @@ void launch_count_arcs(int n, int Q, int64_t S, const StepRec* rec,
                        unsigned long long* total, int grid, cudaStream_t st);
 
 // FP64 mean of a float array, deterministic (fixed blocking and order)
+// over up to 256 blocks; the last of partial's kMeanBlocks words holds the
+// counter of blocks done, which has to be zero at launch
 constexpr int kMeanBlocks = 512;
+inline uint32_t* mean_counter(double* partial) {
+  return reinterpret_cast<uint32_t*>(partial + (kMeanBlocks - 1));
+}
 void launch_mean(const float* x, int64_t count, double* partial /*[kMeanBlocks]*/,
                  double* out, cudaStream_t st);
 
-// adjoint assembly: grad[(n+1)^2] = counts / S * (*grad_mean)
-void launch_grad_assemble(int n, int64_t S, const int32_t* tour,
-                          const unsigned long long* hist, const float* grad_mean,
-                          float* grad, int64_t* hist_out, cudaStream_t st);
+// adjoint assembly: grad[(n+1)^2] = counts / S * (*grad_mean) (float or double)
+int launch_grad(int n, int64_t S, const int32_t* tour, const unsigned long long* hist,
+                const void* grad_mean, bool grad_is_double, float* grad, int64_t* hist_out,
+                cudaStream_t st);
 void launch_backtrack_hist(int n, int64_t S, const void* pred, int pred_dtype,
                            unsigned long long* hist, uint32_t* status,
                            cudaStream_t st);
@@ -388,6 +400,7 @@ struct ReinsertArgs {
   float* value0;
   uint32_t* status;
   uint32_t* dscratch;  // lane kernel with a policy: reinsert_lane_scratch_bytes
+  uint32_t* mean_counter;  // set to zero for the mean that follows, or NULL
   int n_routes;               // route options per day (0: the two-action DP)
   const float* route_cost;    // [T * n_routes]
   const int32_t* route_cap;   // [S * T * n_routes]

@@ -20,9 +20,13 @@ __device__ __forceinline__ float travel(const float* coords, const float* dist,
 __global__ void __launch_bounds__(256) tour_prep_kernel(
     const int32_t* __restrict__ tour, int n, const float* __restrict__ coords,
     const float* __restrict__ dist, TourPrep prep, uint32_t* status,
-    uint32_t* reset_word) {
+    CallCounters counters) {
   __shared__ double red[256];
-  if (threadIdx.x == 0 && reset_word) *reset_word = 0u;
+  if (threadIdx.x == 0) {  // the call's counters, for the kernels that follow
+    if (counters.flagged) *counters.flagged = 0u;
+    if (counters.tiles) *counters.tiles = 0ull;
+    if (counters.mean) *counters.mean = 0u;
+  }
   double acc = 0.0;
   bool bad = false;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -57,9 +61,8 @@ __global__ void __launch_bounds__(256) tour_prep_kernel(
 
 void launch_tour_prep(const int32_t* tour, int n, const float* coords,
                       const float* dist, TourPrep prep, uint32_t* status,
-                      uint32_t* reset_word, cudaStream_t st) {
-  tour_prep_kernel<<<1, 256, 0, st>>>(tour, n, coords, dist, prep, status,
-                                      reset_word);
+                      CallCounters counters, cudaStream_t st) {
+  tour_prep_kernel<<<1, 256, 0, st>>>(tour, n, coords, dist, prep, status, counters);
 }
 
 // ----------------------------------------------------------- arc counting
@@ -99,42 +102,86 @@ void launch_count_arcs(int n, int Q, int64_t S, const StepRec* rec,
 }
 
 // ------------------------------------------------------------- FP64 mean
-// Two passes with a fixed blocking: block b sums its contiguous chunk with a
-// fixed per-thread order and a fixed tree, then one block sums the partials.
-// The result does not depend on scheduling (bit-reproducible).
-__global__ void __launch_bounds__(256) mean_partial_kernel(
-    const float* __restrict__ x, int64_t count, double* partial) {
-  __shared__ double red[256];
-  const int64_t chunk = (count + gridDim.x - 1) / gridDim.x;
-  const int64_t lo = blockIdx.x * chunk;
-  const int64_t hi = min(count, lo + chunk);
+// Eight values as the pair of floats (their rounded sum, the exact sum of its
+// rounding errors by Knuth's two-sum) and then one FP64 number: exact for
+// values within 2^20 of each other, so the sum of any group is what FP64
+// additions give.  GB300 has few FP64 units (a conversion and an addition per
+// value took 48 us for 1,025 x 10^4 values; 0.25 of each per value here).
+__device__ __forceinline__ double sum8(const float* v) {
+  float hi = v[0], lo = 0.f;
+#pragma unroll
+  for (int k = 1; k < 8; ++k) {
+    const float s = __fadd_rn(hi, v[k]);
+    const float t = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(v[k], t)));
+    hi = s;
+  }
+  if (fabsf(hi) <= 3.0e38f) return (double)hi + (double)lo;
+  double acc = 0.0;  // an infinity, a NaN or an overflow of the float sum
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc += (double)v[k];
+  return acc;
+}
+
+// sum of x[lo .. hi) over the CTA's 256 threads, in a fixed order (every
+// thread takes x[lo + thread + 256 j]; the result is valid in thread 0)
+__device__ double block_sum(const float* __restrict__ x, int64_t lo, int64_t hi, double* red) {
   double acc = 0.0;
-  for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) acc += (double)x[k];
+  int64_t k = lo + threadIdx.x;
+  for (; k + 7 * 256 < hi; k += 8 * 256) {
+    float v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = x[k + j * 256];
+    acc += sum8(v);
+  }
+  for (; k < hi; k += 256) acc += (double)x[k];
   red[threadIdx.x] = acc;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+  for (int w = 128; w > 0; w >>= 1) {
     if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
+  return red[0];
 }
 
-__global__ void __launch_bounds__(kMeanBlocks) mean_final_kernel(
-    const double* __restrict__ partial, int64_t count, double* out) {
-  __shared__ double red[kMeanBlocks];
-  red[threadIdx.x] = partial[threadIdx.x];
-  __syncthreads();
-  for (int w = kMeanBlocks / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+// One launch: block b sums its contiguous chunk, the block that finishes last
+// (counter, zero at launch) the partial sums in their order, so the result
+// does not depend on scheduling (bit-reproducible).  One block needs no
+// counter.
+__global__ void __launch_bounds__(256) mean_kernel(const float* __restrict__ x, int64_t count,
+                                                   double* partial, uint32_t* counter, double* out) {
+  __shared__ double red[256];
+  __shared__ bool last;
+  const int64_t chunk = (count + gridDim.x - 1) / gridDim.x;
+  const int64_t lo = blockIdx.x * chunk;
+  double total = block_sum(x, lo, min(count, lo + chunk), red);
+  if (gridDim.x > 1) {
+    if (threadIdx.x == 0) {
+      partial[blockIdx.x] = total;
+      __threadfence();
+      last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
     __syncthreads();
+    if (!last) return;
+    __threadfence();
+    red[threadIdx.x] = threadIdx.x < gridDim.x ? __ldcg(partial + threadIdx.x) : 0.0;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+      __syncthreads();
+    }
+    total = red[0];
   }
-  if (threadIdx.x == 0) *out = count > 0 ? red[0] / (double)count : 0.0;
+  if (threadIdx.x == 0) *out = count > 0 ? total / (double)count : 0.0;
 }
 
+// up to 4,096 values a block, at most 256 blocks (the counter sits behind the
+// partial sums: mean_counter)
 void launch_mean(const float* x, int64_t count, double* partial, double* out,
                  cudaStream_t st) {
-  mean_partial_kernel<<<kMeanBlocks, 256, 0, st>>>(x, count, partial);
-  mean_final_kernel<<<1, kMeanBlocks, 0, st>>>(partial, count, out);
+  const int64_t blocks = (count + 4095) / 4096;
+  const int grid = blocks < 1 ? 1 : (int)imin64(blocks, 256);
+  mean_kernel<<<grid, 256, 0, st>>>(x, count, partial, mean_counter(partial), out);
 }
 
 // ------------------------------------------------------------------ adjoint
@@ -194,32 +241,70 @@ void launch_backtrack_hist(int n, int64_t S, const void* pred, int pred_dtype,
         n, S, (const int32_t*)pred, hist, status);
 }
 
-__global__ void zero_kernel(float* g, int64_t count) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < count;
-       k += (int64_t)gridDim.x * blockDim.x)
-    g[k] = 0.f;
-}
-
 // Each route p+1..i uses (0,s_{p+1}), (s_k,s_{k+1}) for p+1 <= k < i and
 // (s_i,0).  Position k either ends its route (arc (s_k,0)) or continues to
-// s_{k+1}: continue(k) = counted scenarios - ends(k).  The arcs touched by
-// different positions are distinct because the tour is a permutation.
-__global__ void grad_scatter_kernel(int n, int64_t S, const int32_t* __restrict__ tour,
-                                    const unsigned long long* __restrict__ hist,
-                                    const float* __restrict__ grad_mean,
-                                    float* __restrict__ grad, int64_t* hist_out) {
-  const double scale = (double)__ldg(grad_mean) / (double)S;
+// s_{k+1}: continue(k) = counted scenarios - ends(k).  Every entry of the
+// matrix is written once: a block inverts the tour in shared memory (position
+// of each customer, 0 where the tour does not hold it) and takes whole rows.
+// GT: the type of the incoming gradient, taken as a float.
+template <typename GT>
+__global__ void __launch_bounds__(256) grad_kernel(int n, int64_t S, const int32_t* __restrict__ tour,
+                                                   const unsigned long long* __restrict__ hist,
+                                                   const GT* __restrict__ grad_mean,
+                                                   float* __restrict__ grad, int64_t* hist_out) {
+  extern __shared__ int32_t pos[];  // [n + 1], 1-based
+  const int m = n + 1;
+  for (int k = threadIdx.x; k < m; k += blockDim.x) pos[k] = 0;
+  __syncthreads();
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const int sk = __ldg(tour + k);
+    if (sk >= 1 && sk <= n) pos[sk] = k + 1;  // (an invalid entry is flagged by tour_prep)
+  }
+  __syncthreads();
+  const bool any = n > 0 && S > 0;
+  const double scale = any ? (double)(float)__ldg(grad_mean) / (double)S : 0.0;
+  const unsigned long long used = any ? hist[2 * n] : 0ull;
+  for (int a = blockIdx.x; a < m; a += gridDim.x) {
+    const int pa = pos[a];
+    const unsigned long long ends = any && pa ? hist[n + pa - 1] : 0ull;
+    for (int b = threadIdx.x; b < m; b += blockDim.x) {
+      const int pb = pos[b];
+      float g = 0.f;
+      if (any) {
+        if (a == 0) {
+          if (pb) g = (float)((double)hist[pb - 1] * scale);
+        } else if (pa) {
+          if (b == 0) g = (float)((double)ends * scale);
+          else if (pb == pa + 1) g = (float)((double)(used - ends) * scale);
+        }
+      }
+      grad[(size_t)a * m + b] = g;
+    }
+  }
+  if (hist_out && blockIdx.x == 0 && any)
+    for (int k = threadIdx.x; k < 2 * n; k += blockDim.x) hist_out[k] = (int64_t)hist[k];
+}
+
+// The same over a zeroed matrix, for tours whose inverse does not fit shared
+// memory (n > 58,000): position k writes its own arcs, which are distinct
+// because the tour is a permutation.
+template <typename GT>
+__global__ void __launch_bounds__(256) grad_scatter_kernel(int n, int64_t S,
+                                                           const int32_t* __restrict__ tour,
+                                                           const unsigned long long* __restrict__ hist,
+                                                           const GT* __restrict__ grad_mean,
+                                                           float* __restrict__ grad, int64_t* hist_out) {
+  const double scale = (double)(float)__ldg(grad_mean) / (double)S;
   const unsigned long long used = hist[2 * n];
   const int m = n + 1;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n;
-       k += gridDim.x * blockDim.x) {
-    int sk = __ldg(tour + k);
-    if (sk < 1 || sk > n) continue;  // invalid tour entry (flagged by tour_prep)
-    unsigned long long st = hist[k], en = hist[n + k];
-    grad[(size_t)0 * m + sk] = (float)((double)st * scale);
-    grad[(size_t)sk * m + 0] = (float)((double)en * scale);
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int sk = __ldg(tour + k);
+    if (sk < 1 || sk > n) continue;
+    const unsigned long long st = hist[k], en = hist[n + k];
+    grad[(size_t)sk] = (float)((double)st * scale);
+    grad[(size_t)sk * m] = (float)((double)en * scale);
     if (k + 1 < n) {
-      int sn = __ldg(tour + k + 1);
+      const int sn = __ldg(tour + k + 1);
       if (sn >= 1 && sn <= n) grad[(size_t)sk * m + sn] = (float)((double)(used - en) * scale);
     }
     if (hist_out) {
@@ -229,17 +314,35 @@ __global__ void grad_scatter_kernel(int n, int64_t S, const int32_t* __restrict_
   }
 }
 
-void launch_grad_assemble(int n, int64_t S, const int32_t* tour,
-                          const unsigned long long* hist, const float* grad_mean,
-                          float* grad, int64_t* hist_out, cudaStream_t st) {
-  int64_t cnt = (int64_t)(n + 1) * (n + 1);
-  int g1 = (int)imin64((cnt + 255) / 256, 4 * num_sms());
-  zero_kernel<<<g1, 256, 0, st>>>(grad, cnt);
-  if (n > 0 && S > 0) {
-    int g2 = (n + 255) / 256;
-    grad_scatter_kernel<<<g2, 256, 0, st>>>(n, S, tour, hist, grad_mean, grad,
-                                            hist_out);
+namespace {
+template <typename GT>
+int launch_grad_t(int n, int64_t S, const int32_t* tour, const unsigned long long* hist,
+                  const GT* grad_mean, float* grad, int64_t* hist_out, cudaStream_t st) {
+  const size_t smem = (size_t)(n + 1) * 4;
+  if (smem > 227 * 1024) {
+    const cudaError_t e = cudaMemsetAsync(grad, 0, (size_t)(n + 1) * (size_t)(n + 1) * sizeof(float), st);
+    if (e != cudaSuccess) return (int)e;
+    if (S > 0)
+      grad_scatter_kernel<GT><<<(n + 255) / 256, 256, 0, st>>>(n, S, tour, hist, grad_mean, grad, hist_out);
+    return (int)cudaGetLastError();
   }
+  if (smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(grad_kernel<GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return (int)e;
+  }
+  const int grid = (int)imin64(n + 1, 4 * (int64_t)num_sms());
+  grad_kernel<GT><<<grid, 256, smem, st>>>(n, S, tour, hist, grad_mean, grad, hist_out);
+  return (int)cudaGetLastError();
+}
+}  // namespace
+
+int launch_grad(int n, int64_t S, const int32_t* tour, const unsigned long long* hist,
+                const void* grad_mean, bool grad_is_double, float* grad, int64_t* hist_out,
+                cudaStream_t st) {
+  return grad_is_double
+             ? launch_grad_t(n, S, tour, hist, (const double*)grad_mean, grad, hist_out, st)
+             : launch_grad_t(n, S, tour, hist, (const float*)grad_mean, grad, hist_out, st);
 }
 
 }  // namespace sdp
@@ -299,16 +402,8 @@ void launch_batch_prep(const BatchPrepArgs& a, int B, cudaStream_t st) {
 __global__ void __launch_bounds__(256) batch_mean_kernel(const float* __restrict__ costs,
                                                          int64_t S, double* means) {
   __shared__ double red[256];
-  const float* x = costs + (int64_t)blockIdx.x * S;
-  double acc = 0.0;
-  for (int64_t k = threadIdx.x; k < S; k += blockDim.x) acc += (double)x[k];
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) means[blockIdx.x] = red[0] / (double)S;
+  const double total = block_sum(costs + (int64_t)blockIdx.x * S, 0, S, red);
+  if (threadIdx.x == 0) means[blockIdx.x] = total / (double)S;
 }
 
 void launch_batch_means(const float* costs, int B, int64_t S, double* means, cudaStream_t st) {
