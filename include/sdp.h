@@ -309,6 +309,23 @@ int sdp_split_backward(const sdp_split_args* fwd, const void* pred,
                        const float* grad_mean, float* grad_dist,
                        int64_t* route_hist_out, void* stream);
 
+/* Costs and route counts of one evaluation, for a training step: what
+ * sdp_split_eval returns (no predecessors), and in routes_out [2n+1] how many
+ * scenarios start a route at position k ([k]), end one there ([n+k]), and how
+ * many were counted ([2n], those with a feasible split) -- the counts that
+ * sdp_split_backward recomputes.  Runs where the fused adjoint kernel does
+ * (hard capacity, device demands, demand rows of up to 512 staged bytes):
+ * sdp_split_routes_workspace_bytes(a) is its workspace, 0 where it does not
+ * run (SDP_ERR_UNSUPPORTED).  cost_out may be NULL (size the workspace with
+ * the same cost_out as the call).
+ * sdp_split_grad_from_routes turns them into d mean / d dist [(n+1)^2] times
+ * *grad_mean (a device float, or a double that is rounded to float first). */
+size_t sdp_split_routes_workspace_bytes(const sdp_split_args* a);
+int sdp_split_eval_routes(const sdp_split_args* a, uint64_t* routes_out, void* stream);
+int sdp_split_grad_from_routes(int32_t n, int64_t S, const int32_t* tour, const uint64_t* routes,
+                               const void* grad_mean, int32_t grad_is_double, float* grad_dist,
+                               void* stream);
+
 /* -------------------------------------------------------- batched Split */
 /* The Split of Eq. eqdpA for B giant tours of uneven length, S scenarios
  * each (the candidate evaluations Tables cand_cvrp / gpu_dsirp count), run

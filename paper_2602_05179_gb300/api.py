@@ -106,6 +106,9 @@ def _load():
             "sdp_split_fleet_eval": ([P, i32, P, P, P], i32),
             "sdp_split_backward_workspace_bytes": ([P], sz),
             "sdp_split_backward": ([P, P, P, P, P, P], i32),
+            "sdp_split_routes_workspace_bytes": ([P], sz),
+            "sdp_split_eval_routes": ([P, P, P], i32),
+            "sdp_split_grad_from_routes": ([i32, i64, P, P, P, i32, P, P], i32),
             "sdp_reinsert_workspace_bytes": ([P], sz),
             "sdp_reinsert_eval": ([P, P], i32),
             "sdp_set_profile_events": ([P, P], i32),
@@ -449,27 +452,72 @@ class SplitMeanCost(torch.autograd.Function):
     forward(dist [n+1, n+1] fp32 CUDA, tour, demands, Q, keep_pred=False)
     returns the FP64 scenario mean (0-d); backward returns
     d mean / d dist = (1/S) x arc-usage counts of the optimal splits (the
-    cost is piecewise linear in dist), computed by the library's backtrack
-    kernel from stored predecessors (keep_pred=True) or by the fused
-    forward + on-chip backtrack kernel."""
+    cost is piecewise linear in dist).  Where a gradient is wanted and the
+    fused kernel applies, the forward counts the routes while it evaluates
+    and the backward only assembles the matrix; otherwise the counts come
+    from stored predecessors (keep_pred=True) by the library's backtrack
+    kernel or are recomputed by the fused forward + backtrack kernel."""
+
+    @classmethod
+    def apply(cls, dist, tour, demands, Q, keep_pred=False):
+        # forward runs with gradients off: whether one is wanted is seen here
+        return super().apply(dist, tour, demands, Q, keep_pred, torch.is_grad_enabled())
 
     @staticmethod
-    def forward(ctx, dist, tour, demands, Q, keep_pred=False):
-        r = split_eval(tour, Q, demands, dist=dist, preds="u16" if keep_pred else None)
-        ctx.save_for_backward(dist, tour, demands)
+    def forward(ctx, dist, tour, demands, Q, keep_pred=False, grad_enabled=False):
+        r = routes = None
+        if grad_enabled and ctx.needs_input_grad[0] and not keep_pred:
+            r, routes = _split_mean_routes(tour, Q, demands, dist)
+        if r is None:
+            r = split_eval(tour, Q, demands, dist=dist, preds="u16" if keep_pred else None)
+        ctx.save_for_backward(dist, tour, demands, routes)
         ctx.Q = int(Q)
         ctx.pred = r["pred"]
         return r["mean"]
 
     @staticmethod
     def backward(ctx, grad_out):
-        dist, tour, demands = ctx.saved_tensors
+        dist, tour, demands, routes = ctx.saved_tensors
+        if routes is not None:
+            return (_grad_from_routes(tour, int(demands.shape[0]), routes, grad_out),
+                    None, None, None, None, None)
         pred = ctx.pred
         if pred is not None and pred.dtype != torch.int16:
             pred = pred.view(torch.int16)
         g, _ = split_backward(tour, ctx.Q, demands, dist, grad_out, pred=pred,
                               pred_dtype="u16" if pred is not None else None)
-        return g, None, None, None, None
+        return g, None, None, None, None, None
+
+
+def _split_mean_routes(tour, Q, demands, dist):
+    """split_eval's mean and the route counts int64 [2n + 1] of the optimal
+    splits from one kernel; (None, None) where no kernel returns both."""
+    lib = _load()
+    n, dev = int(tour.numel()), tour.device
+    a = _split_struct(tour, Q, demands, None, dist, None, None, 0, "auto", None, 0, 0)
+    nbytes = lib.sdp_split_routes_workspace_bytes(ctypes.byref(a))
+    if nbytes == 0:
+        return None, None
+    mean = torch.empty((), dtype=torch.float64, device=dev)
+    routes = torch.empty(2 * n + 1, dtype=torch.int64, device=dev)
+    ws = _workspace(nbytes, dev)
+    a.mean_out = mean.data_ptr()
+    a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
+    _check(lib.sdp_split_eval_routes(ctypes.byref(a), routes.data_ptr(), _stream(None)))
+    return {"pred": None, "mean": mean}, routes
+
+
+def _grad_from_routes(tour, S, routes, grad_mean):
+    """d mean / d dist (fp32 [n+1, n+1]) times grad_mean from route counts."""
+    n = int(tour.numel())
+    grad = torch.empty((n + 1, n + 1), dtype=torch.float32, device=tour.device)
+    gm = grad_mean
+    if gm.device != tour.device or gm.dtype not in (torch.float32, torch.float64):
+        gm = gm.to(device=tour.device, dtype=torch.float32)
+    _check(_load().sdp_split_grad_from_routes(n, S, tour.data_ptr(), routes.data_ptr(), gm.data_ptr(),
+                                              1 if gm.dtype == torch.float64 else 0, grad.data_ptr(),
+                                              _stream(None)))
+    return grad
 
 
 REINSERT_ALGOS = {"auto": 0, "warp": 1, "lane": 2}

@@ -327,7 +327,7 @@ SplitWs carve_split(const sdp_split_args* a, void* base, bool backward) {
 }
 
 int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
-                   unsigned long long* hist, cudaStream_t st);
+                   unsigned long long* hist, cudaStream_t st, bool hist_and_cost = false);
 
 // Copy stream and events of the host-demand pipeline, made once per device on
 // first use and kept for the life of the process.
@@ -463,14 +463,14 @@ int check_ws(void* ws, size_t have, size_t need) {
 // Runs the chosen DP kernel over all S, then recomputes the scenarios it
 // flagged (one warp each where its rows fit split_rescue.cu's shared memory;
 // else the plain kernel over the flagged list), or runs the PLAIN kernel over
-// all S.
+// all S.  With route counts (hist) costs are written only if hist_and_cost.
 int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
-                   unsigned long long* hist, cudaStream_t st) {
+                   unsigned long long* hist, cudaStream_t st, bool hist_and_cost) {
   int algo = resolve_algo(a);
   if ((algo == SDP_ALGO_STREAM || algo == SDP_ALGO_PIPE) && hist)
     algo = SDP_ALGO_DEQUE;  // the fused adjoint is DEQUE's
   const int sms = num_sms();
-  float* cost = hist ? nullptr : a->cost_out;
+  float* cost = hist && !hist_and_cost ? nullptr : a->cost_out;
   void* pred = hist ? nullptr : a->pred_out;
   if (algo == SDP_ALGO_STREAM) {
     StreamArgs sa{};
@@ -512,7 +512,7 @@ int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
     SplitDequeArgs d{};
     d.n = a->n; d.Q = a->Q; d.S = a->S;
     d.rec = w.prep.rec; d.cols = w.prep.cols; d.Dn = w.prep.Dn;
-    d.demands = a->demands; d.cost = nullptr; d.pred = nullptr; d.pred_dtype = a->pred_dtype;
+    d.demands = a->demands; d.cost = cost; d.pred = nullptr; d.pred_dtype = a->pred_dtype;
     d.hist = hist; d.fb_list = w.fb_list; d.fb_count = w.fb_count; d.status = status;
     note_launch(adj_warps, sms);
     prof_begin(st);
@@ -970,20 +970,80 @@ int sdp_split_backward(const sdp_split_args* args, const void* pred, const float
   if (rc) return rc;
   const SplitWs w = carve_split(fwd, fwd->workspace, true);
   const int n = fwd->n;
-  cudaError_t e = cudaMemsetAsync(w.hist, 0, sizeof(unsigned long long) * (2 * (size_t)n + 1), st);
-  if (e != cudaSuccess) return cuda_fail(e, "memset hist");
-  if (n > 0 && fwd->S > 0) {
-    if (pred) {
+  if (n > 0 && fwd->S > 0 && !pred) {
+    launch_tour_prep(fwd->tour, n, fwd->coords, fwd->dist, w.prep, status,
+                     {w.fb_count, w.counter, nullptr, w.hist}, st);
+    rc = run_split_core(fwd, w, status, w.hist, st);
+    if (rc) return rc;
+  } else {
+    const cudaError_t e = cudaMemsetAsync(w.hist, 0, sizeof(unsigned long long) * (2 * (size_t)n + 1), st);
+    if (e != cudaSuccess) return cuda_fail(e, "memset hist");
+    if (n > 0 && fwd->S > 0)
       launch_backtrack_hist(n, fwd->S, pred, fwd->pred_dtype, w.hist, status, st);
-    } else {
-      launch_tour_prep(fwd->tour, n, fwd->coords, fwd->dist, w.prep, status,
-                       {w.fb_count, w.counter, nullptr}, st);
-      rc = run_split_core(fwd, w, status, w.hist, st);
-      if (rc) return rc;
-    }
   }
   const int ge = launch_grad(n, fwd->S, fwd->tour, w.hist, grad_mean, false, grad_dist, route_hist_out, st);
   if (ge) return cuda_fail((cudaError_t)ge, "backward launch");
+  return SDP_OK;
+}
+
+// ------------------------------------------- costs and route counts together
+size_t sdp_split_routes_workspace_bytes(const sdp_split_args* a) {
+  if (!a || a->n < 1 || a->S < 1 || a->Q <= 0 || a->capacity_mode != SDP_CAPACITY_HARD ||
+      is_host_ptr(a->demands) || adjoint_tmem_warps(a) < 1)
+    return 0;
+  return carve_split(a, nullptr, true).bytes + (a->cost_out ? 0 : sizeof(float) * (size_t)a->S);
+}
+
+int sdp_split_eval_routes(const sdp_split_args* args, uint64_t* routes_out, void* stream) {
+  int rc = check_split(args, false);
+  if (rc) return rc;
+  if (args->cost_out && !is_device_ptr(args->cost_out))
+    return fail(SDP_ERR_INVALID_ARG, "cost_out must be a device pointer");
+  if (!is_device_ptr(routes_out)) return fail(SDP_ERR_INVALID_ARG, "routes_out must be a device pointer");
+  if (args->pred_out)
+    return fail(SDP_ERR_INVALID_ARG, "sdp_split_eval_routes returns route counts, not pred_out");
+  const size_t need = sdp_split_routes_workspace_bytes(args);
+  if (need == 0)
+    return fail(SDP_ERR_UNSUPPORTED, "this shape has no kernel that returns costs and route counts together");
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  rc = check_ws(args->workspace, args->workspace_bytes, need);
+  if (rc) return rc;
+  uint32_t* status;
+  rc = status_ptr(&status);
+  if (rc) return rc;
+  rc = fault_call();
+  if (rc) return rc;
+  const SplitWs w = carve_split(args, args->workspace, true);
+  sdp_split_args with_cost = *args;
+  const sdp_split_args* a = &with_cost;
+  if (!a->cost_out)
+    with_cost.cost_out = reinterpret_cast<float*>(static_cast<unsigned char*>(args->workspace) + w.bytes);
+  unsigned long long* routes = reinterpret_cast<unsigned long long*>(routes_out);
+  launch_tour_prep(a->tour, a->n, a->coords, a->dist, w.prep, status,
+                   {w.fb_count, w.counter, mean_counter(w.mean_partial), routes}, st);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "tour_prep launch");
+  rc = run_split_core(a, w, status, routes, st, true);
+  if (rc) return rc;
+  if (a->mean_out) {
+    launch_mean(a->cost_out, a->S, w.mean_partial, a->mean_out, st);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "mean launch");
+  }
+  return SDP_OK;
+}
+
+int sdp_split_grad_from_routes(int32_t n, int64_t S, const int32_t* tour, const uint64_t* routes,
+                               const void* grad_mean, int32_t grad_is_double, float* grad_dist,
+                               void* stream) {
+  if (n < 1 || S < 1) return fail(SDP_ERR_INVALID_ARG, "n and S must be >= 1");
+  if (!is_device_ptr(tour) || !is_device_ptr(routes) || !is_device_ptr(grad_mean) || !is_device_ptr(grad_dist))
+    return fail(SDP_ERR_INVALID_ARG, "tour, routes, grad_mean and grad_dist must be device pointers");
+  const int rc = fault_call();
+  if (rc) return rc;
+  const int e = launch_grad(n, S, tour, reinterpret_cast<const unsigned long long*>(routes), grad_mean,
+                            grad_is_double != 0, grad_dist, nullptr, static_cast<cudaStream_t>(stream));
+  if (e) return cuda_fail((cudaError_t)e, "gradient launch");
   return SDP_OK;
 }
 

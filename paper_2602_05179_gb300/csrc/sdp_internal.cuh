@@ -40,11 +40,12 @@ struct TourPrep {
 // status bits are OR-ed into *status (a per-device __device__ word).
 
 // Counters of a call that its first kernel sets to zero (NULL: none): flagged
-// scenarios, tiles claimed, blocks of the mean done.
+// scenarios, tiles claimed, blocks of the mean done, route counts [2n+1].
 struct CallCounters {
   uint32_t* flagged;
   unsigned long long* tiles;
   uint32_t* mean;
+  unsigned long long* routes = nullptr;
 };
 // one CTA per tour; coords or dist mode
 void launch_tour_prep(const int32_t* tour, int n, const float* coords,
@@ -118,7 +119,7 @@ DequeConfig deque_config_wide(const DequeConfig& c, int n, int Q, int64_t S, boo
 // Fused adjoint and forward with TMEM-staged rows: warps per CTA (16..24)
 // for S scenarios on sms SMs (more than 16 only for a single round), 0 where
 // rows do not fit 16 warps' columns; the [word][lane] delta
-// scratch it needs; the launch (hist set, cost / pred unused).
+// scratch it needs; the launch (hist set, cost optional, pred unused).
 int split_tmem_adj_warps(int n, int Q, int64_t S, int sms);
 size_t split_tmem_adj_scratch_bytes(int n, int Q, int sms);
 int launch_split_tmem_adj(const SplitDequeArgs& a, int warps, uint32_t* dscratch, int sms,
@@ -189,7 +190,7 @@ struct RescueArgs {
   int n_max;                   // longest tour (shared memory per warp: 8..12 (n_max+1) bytes)
   int soft;                    // one tour: soft capacity, beta per unit of route load above Q
   float beta;
-  unsigned long long* hist;    // one tour, hard: route counts [2n+1] instead of costs, or NULL
+  unsigned long long* hist;    // one tour, hard: route counts [2n+1], or NULL
   // one tour
   int n1;
   const uint32_t* fb_list1;    // [*fb_count] scenario ids

@@ -27,6 +27,8 @@ __global__ void __launch_bounds__(256) tour_prep_kernel(
     if (counters.tiles) *counters.tiles = 0ull;
     if (counters.mean) *counters.mean = 0u;
   }
+  if (counters.routes)
+    for (int k = threadIdx.x; k < 2 * n + 1; k += blockDim.x) counters.routes[k] = 0ull;
   double acc = 0.0;
   bool bad = false;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {

@@ -1179,14 +1179,17 @@ __global__ void __launch_bounds__(512 + 32 * XW, 1) split_tmem_kernel(SplitDeque
   if (warp == 0) tmem_dealloc(tmem_base, 512);
 }
 
-// Fused adjoint with TMEM staging: the forward DP of split_tmem_kernel
-// (cost not stored), i - pred(i) of each position packed into the warp's
-// slot of a [word][lane] global scratch (one coalesced 128-byte store every
+// Fused adjoint with TMEM staging: the forward DP of split_tmem_kernel (costs
+// stored where a.cost is set: a training step's forward and its route counts
+// from one pass, 113 us at n = 300, S = 10^5 where the forward by PIPE and then
+// this kernel took 105 + 112), i - pred(i) of each position packed into the
+// warp's slot of a [word][lane] global scratch (one coalesced 128-byte store every
 // 4 uint8 / 2 uint16 positions), then each lane walks its own scenario's
 // optimal routes back from position n and counts route starts / ends in
 // shared-memory histograms.  The CTA holds blockDim.x / 32 = 16..24 warps:
 // more than 16 when that many take every tile in one round where 16 would
-// need two (a second, partly empty round costs a whole row's time).  Warp w
+// need two (a second, partly empty round costs a whole row's time), and fewer
+// where they already cover the tiles on every SM.  Warp w
 // holds its tile in TMEM lane quadrant w % 4, column block w / 4 of
 // cols_per_warp.
 template <typename QT, int MAXT>
@@ -1231,6 +1234,7 @@ __global__ void __launch_bounds__(MAXT, 1) split_tmem_adj_kernel(SplitDequeArgs 
                          (uint32_t)((warp >> 2) * cols_per_warp);
   uint32_t* dl = dscratch + ((int64_t)blockIdx.x * nwarps + warp) * dwords * 32 + lane;
 
+  const double Dn = a.cost ? *a.Dn : 0.0;
   bool neg = false;
   uint32_t any_inf = 0, any_fb = 0;
   const int64_t wstride = (int64_t)gridDim.x * nwarps;
@@ -1258,6 +1262,8 @@ __global__ void __launch_bounds__(MAXT, 1) split_tmem_adj_kernel(SplitDequeArgs 
     if (bad) {
       const uint32_t k = atomicAdd(a.fb_count, 1u);
       a.fb_list[k] = (uint32_t)(s0 + lane);
+    } else if (a.cost && valid) {
+      a.cost[s0 + lane] = first_inf <= (uint32_t)n ? CUDART_INF_F : (float)((double)K + Dn);
     }
     any_inf |= tf.inf_rows;
     any_fb |= __ballot_sync(0xffffffffu, bad);
@@ -1835,9 +1841,13 @@ int launch_adj_t(const SplitDequeArgs& a, int nw, uint32_t* dscratch, int sms,
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
   const int64_t tiles = (a.S + 31) / 32;
-  const int64_t ctas = (tiles + nw - 1) / nw;
+  // few tiles: on every SM, a few warps each (831 tiles of n = 183 on 52 CTAs of
+  // 16 warps took 62 us, on 139 of 6 50)
+  const int64_t share = (tiles + sms - 1) / sms;
+  const int warps = (int)(share < nw ? share : nw);
+  const int64_t ctas = (tiles + warps - 1) / warps;
   const int grid = (int)(ctas < sms ? ctas : sms);
-  k<<<grid, 32 * nw, smem, st>>>(a, tiles, tmem_cols_per_warp(nw), dscratch);
+  k<<<grid, 32 * warps, smem, st>>>(a, tiles, tmem_cols_per_warp(nw), dscratch);
   return (int)cudaGetLastError();
 }
 }  // namespace

@@ -48,8 +48,8 @@ size_t rescue_per_warp(int n_max, bool soft, bool hist) {
   return (size_t)(8 + (soft ? 4 : 0) + (hist ? 4 : 0)) * ((size_t)n_max + 1);
 }
 
-// PT: predecessor type; HIST: count route starts / ends into a.hist instead of
-// writing costs
+// PT: predecessor type; HIST: count route starts / ends into a.hist (costs only
+// where a.cost is set)
 template <typename PT, bool BATCH, bool SOFT, bool HIST>
 __global__ void __launch_bounds__(kRescueMaxWarps * 32) split_rescue_kernel(RescueArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(kRescueMaxWarps * 32) split_rescue_kernel(Resc
         }
         atomicAdd(&a.hist[2 * n], 1ull);
       }
-    } else if (lane == 0) {
+    }
+    if (lane == 0 && (!HIST || a.cost)) {
       const float c = inf ? CUDART_INF_F : (float)((double)Kn + Dn);
       if (BATCH) a.costs[out] = c;
       else a.cost[out] = c;
