@@ -39,6 +39,7 @@
 #include <math.h>
 #include <math_constants.h>
 
+#include "dependent.cuh"
 #include "sdp_internal.cuh"
 
 namespace sdp {
@@ -70,6 +71,7 @@ struct Flag {
 template <bool TABLE, bool UNIT, int RK>
 __global__ void __launch_bounds__(kChainMaxWarps * 32, 1) reinsert_chain_kernel(ReinsertArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  dep_launch();
   if (a.mean_counter && blockIdx.x == 0 && threadIdx.x == 0) *a.mean_counter = 0u;
   constexpr int CW = RK / 4;                // capacity words per scenario-day
   constexpr int DW = RK > 0 ? RK : 1;       // daily costs per day

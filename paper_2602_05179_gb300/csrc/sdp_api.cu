@@ -472,6 +472,8 @@ int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
   const int sms = num_sms();
   float* cost = hist && !hist_and_cost ? nullptr : a->cost_out;
   void* pred = hist ? nullptr : a->pred_out;
+  // chunks of host demands come behind a copy, profiled kernels behind an event
+  const int after_prep = w.stage_rows == 0 && !g_prof_start;
   if (algo == SDP_ALGO_STREAM) {
     StreamArgs sa{};
     sa.n = a->n; sa.Q = a->Q; sa.S = a->S;
@@ -497,6 +499,7 @@ int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
     pa.demands = a->demands; pa.cost = cost; pa.pred = pred; pa.pred_dtype = a->pred_dtype;
     pa.qt = w.qt; pa.stride = pipe_row_stride(a->n, a->Q); pa.counter = w.counter;
     pa.fb_count = w.fb_count; pa.fb_list1 = w.fb_list; pa.status = status;
+    pa.after_prep = after_prep;
     pa.soft = a->capacity_mode == SDP_CAPACITY_SOFT ? 1 : 0; pa.beta = a->overload_penalty;
     const uint64_t stall = fault_stall_ns();
     pa.wait_ns = stall ? stall : kWaitLimitNs;
@@ -514,6 +517,7 @@ int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
     d.rec = w.prep.rec; d.cols = w.prep.cols; d.Dn = w.prep.Dn;
     d.demands = a->demands; d.cost = cost; d.pred = nullptr; d.pred_dtype = a->pred_dtype;
     d.hist = hist; d.fb_list = w.fb_list; d.fb_count = w.fb_count; d.status = status;
+    d.after_prep = after_prep;
     note_launch(adj_warps, sms);
     prof_begin(st);
     const int e = launch_split_tmem_adj(d, adj_warps, w.dscratch, sms, st);

@@ -90,6 +90,7 @@ struct SplitDequeArgs {
   uint32_t* status;
   int soft;             // soft capacity: beta per unit of route load above Q
   float beta;
+  int after_prep = 0;          // the stream's previous operation is the tour preparation
 };
 struct DequeConfig {
   int warps;        // warps per CTA
@@ -309,6 +310,7 @@ struct PipeArgs {
   uint32_t* status;
   uint64_t wait_ns;            // a bounded wait gives up after this
   int stall;                   // fault injection (tests): producers publish no tile
+  int after_prep;              // the stream's previous operation is the tour preparation
 };
 bool pipe_supported(int n, int Q);
 // bytes per tour-ordered slot row: n narrowed demands (uint8 for Q <= 254,

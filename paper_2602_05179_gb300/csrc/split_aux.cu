@@ -1,5 +1,6 @@
 // split_aux.cu -- tour preparation, feasible-arc counting, the deterministic
 // FP64 scenario mean, and the Split adjoint's backtrack / gradient assembly.
+#include "dependent.cuh"
 #include "sdp_internal.cuh"
 
 namespace sdp {
@@ -22,6 +23,7 @@ __global__ void __launch_bounds__(256) tour_prep_kernel(
     const float* __restrict__ dist, TourPrep prep, uint32_t* status,
     CallCounters counters) {
   __shared__ double red[256];
+  dep_launch();
   if (threadIdx.x == 0) {  // the call's counters, for the kernels that follow
     if (counters.flagged) *counters.flagged = 0u;
     if (counters.tiles) *counters.tiles = 0ull;
@@ -127,7 +129,7 @@ __device__ __forceinline__ double sum8(const float* v) {
 
 // sum of x[lo .. hi) over the CTA's 256 threads, in a fixed order (every
 // thread takes x[lo + thread + 256 j]; the result is valid in thread 0)
-__device__ double block_sum(const float* __restrict__ x, int64_t lo, int64_t hi, double* red) {
+__device__ double block_sum(const float* x, int64_t lo, int64_t hi, double* red) {
   double acc = 0.0;
   int64_t k = lo + threadIdx.x;
   for (; k + 7 * 256 < hi; k += 8 * 256) {
@@ -150,10 +152,10 @@ __device__ double block_sum(const float* __restrict__ x, int64_t lo, int64_t hi,
 // (counter, zero at launch) the partial sums in their order, so the result
 // does not depend on scheduling (bit-reproducible).  One block needs no
 // counter.
-__global__ void __launch_bounds__(256) mean_kernel(const float* __restrict__ x, int64_t count,
-                                                   double* partial, uint32_t* counter, double* out) {
+__global__ void __launch_bounds__(256) mean_kernel(const float* x, int64_t count, double* partial, uint32_t* counter, double* out) {
   __shared__ double red[256];
   __shared__ bool last;
+  dep_wait();
   const int64_t chunk = (count + gridDim.x - 1) / gridDim.x;
   const int64_t lo = blockIdx.x * chunk;
   double total = block_sum(x, lo, min(count, lo + chunk), red);
@@ -183,7 +185,7 @@ void launch_mean(const float* x, int64_t count, double* partial, double* out,
                  cudaStream_t st) {
   const int64_t blocks = (count + 4095) / 4096;
   const int grid = blocks < 1 ? 1 : (int)imin64(blocks, 256);
-  mean_kernel<<<grid, 256, 0, st>>>(x, count, partial, mean_counter(partial), out);
+  launch_dependent(true, mean_kernel, grid, 256, 0, st, x, count, partial, mean_counter(partial), out);
 }
 
 // ------------------------------------------------------------------ adjoint
@@ -401,15 +403,16 @@ void launch_batch_prep(const BatchPrepArgs& a, int B, cudaStream_t st) {
 }
 
 // Per-tour FP64 mean of costs[b*S .. b*S+S): one CTA per tour, fixed order.
-__global__ void __launch_bounds__(256) batch_mean_kernel(const float* __restrict__ costs,
-                                                         int64_t S, double* means) {
+__global__ void __launch_bounds__(256) batch_mean_kernel(const float* costs, int64_t S,
+                                                         double* means) {
   __shared__ double red[256];
+  dep_wait();
   const double total = block_sum(costs + (int64_t)blockIdx.x * S, 0, S, red);
   if (threadIdx.x == 0) means[blockIdx.x] = total / (double)S;
 }
 
 void launch_batch_means(const float* costs, int B, int64_t S, double* means, cudaStream_t st) {
-  batch_mean_kernel<<<B, 256, 0, st>>>(costs, S, means);
+  launch_dependent(true, batch_mean_kernel, B, 256, 0, st, costs, S, means);
 }
 
 // Feasible arcs of every (tour, scenario) of a batch.

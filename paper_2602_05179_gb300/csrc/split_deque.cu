@@ -48,6 +48,7 @@
 // chip into shared-memory route start / end histograms.
 #include <math_constants.h>
 
+#include "dependent.cuh"
 #include "sdp_internal.cuh"
 #include "tmem.cuh"
 
@@ -1212,6 +1213,8 @@ __global__ void __launch_bounds__(MAXT, 1) split_tmem_adj_kernel(SplitDequeArgs 
     tmem_alloc(&tmem_base, 512);
     tmem_relinquish();
   }
+  dep_launch();
+  dep_wait();
   StepRec* rec = reinterpret_cast<StepRec*>(smem);
   for (int k = threadIdx.x; k <= n + 1; k += blockDim.x) rec[k] = tmem_rec16<QT>(a.rec[min(k, n - 1)]);
   // from the records in global memory: the shared copy above is not
@@ -1847,8 +1850,7 @@ int launch_adj_t(const SplitDequeArgs& a, int nw, uint32_t* dscratch, int sms,
   const int warps = (int)(share < nw ? share : nw);
   const int64_t ctas = (tiles + warps - 1) / warps;
   const int grid = (int)(ctas < sms ? ctas : sms);
-  k<<<grid, 32 * warps, smem, st>>>(a, tiles, tmem_cols_per_warp(nw), dscratch);
-  return (int)cudaGetLastError();
+  return (int)launch_dependent(a.after_prep != 0, k, grid, 32 * warps, smem, st, a, tiles, tmem_cols_per_warp(nw), dscratch);
 }
 }  // namespace
 

@@ -65,6 +65,7 @@
 #include <math_constants.h>
 
 #include "async_copy.cuh"
+#include "dependent.cuh"
 #include "sdp_internal.cuh"
 
 namespace sdp {
@@ -599,6 +600,8 @@ __global__ void __launch_bounds__(kThreads, 1) split_pipe_kernel(PipeArgs a) {
     slot_ready[threadIdx.x] = 0u;
     slot_free[threadIdx.x] = 0u;
   }
+  dep_launch();
+  dep_wait();
   if (!BATCH) {
     for (int k = threadIdx.x; k < a.n1; k += blockDim.x) {
       const StepRec r = a.rec[k];
@@ -1018,8 +1021,8 @@ int launch_r(const PipeArgs& a, cudaStream_t st) {
   const size_t smem = pipe_smem(a, PRED);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
-  k<<<pipe_grid(a.S, a.B, BATCH), kThreads, smem, st>>>(a);
-  return (int)cudaGetLastError();
+  const int grid = pipe_grid(a.S, a.B, BATCH);
+  return (int)launch_dependent(a.after_prep != 0, k, grid, kThreads, smem, st, a);
 }
 template <typename QT, typename PT, bool PRED, bool BATCH, bool SOFT = false, int NST = 2>
 int launch_k(const PipeArgs& a, cudaStream_t st) {

@@ -31,6 +31,7 @@
 
 #include <algorithm>
 
+#include "dependent.cuh"
 #include "sdp_internal.cuh"
 
 namespace sdp {
@@ -56,6 +57,8 @@ __global__ void __launch_bounds__(kRescueMaxWarps * 32) split_rescue_kernel(Resc
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   const int wpb = blockDim.x >> 5;
+  dep_launch();
+  dep_wait();
   const int64_t nwork = (int64_t)(*a.fb_count);
   const int64_t nw = (int64_t)gridDim.x * wpb;
   constexpr int kArrays = 2 + (SOFT ? 1 : 0) + (HIST ? 1 : 0);
@@ -241,8 +244,7 @@ int launch_r(const RescueArgs& a, int wpb, size_t smem, int grid, cudaStream_t s
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
   }
-  k<<<grid, wpb * 32, smem, st>>>(a);
-  return (int)cudaGetLastError();
+  return (int)launch_dependent(false, k, grid, wpb * 32, smem, st, a);
 }
 
 }  // namespace
