@@ -149,38 +149,26 @@ bool is_device_ptr(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// The address under which the current device reads p: device or managed
-// memory as is, page-locked host memory mapped for the device through its
-// device pointer; NULL for memory the device cannot read.
-const void* device_readable(const void* p) {
-  if (!p) return nullptr;
+// Where demands lie: the address under which the current device reads them
+// (device or managed memory as is, page-locked host memory mapped for the
+// device through its device pointer, NULL for memory the device cannot read),
+// and whether that is page-locked host memory.  Asked of the driver once per
+// call and passed on: a query takes about 0.15 us.
+struct Demands {
+  const int32_t* ptr = nullptr;
+  bool host = false;
+};
+Demands demands_of(const int32_t* p) {
+  Demands d;
+  if (!p) return d;
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
-    return nullptr;
+    return d;
   }
-  if (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) return p;
-  if (at.type == cudaMemoryTypeHost) return at.devicePointer;
-  return nullptr;
-}
-
-// True for page-locked host memory (the device reads it over the host link).
-bool is_host_ptr(const void* p) {
-  if (!p) return false;
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return at.type == cudaMemoryTypeHost;
-}
-
-// The arguments with demands replaced by their device-readable address.
-sdp_split_args with_readable_demands(const sdp_split_args* a) {
-  sdp_split_args b = *a;
-  if (a->demands)
-    b.demands = static_cast<const int32_t*>(device_readable(a->demands));
-  return b;
+  if (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) d.ptr = p;
+  if (at.type == cudaMemoryTypeHost) d = {static_cast<const int32_t*>(at.devicePointer), true};
+  return d;
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -233,12 +221,12 @@ bool soft_deque_ok(const sdp_split_args* a) {
          (int64_t)a->n * (a->Q <= 254 ? 1 : 2) <= 512;
 }
 
-int resolve_algo(const sdp_split_args* a);
+int resolve_algo(const sdp_split_args* a, bool host);
 
 // The fused adjoint runs on the TMEM-staged deque kernel when the forward
 // would take DEQUE in its default shape and a row fits the tensor memory.
-int adjoint_tmem_warps(const sdp_split_args* a) {
-  const int algo = resolve_algo(a);
+int adjoint_tmem_warps(const sdp_split_args* a, bool host) {
+  const int algo = resolve_algo(a, host);
   if (algo != SDP_ALGO_DEQUE && algo != SDP_ALGO_STREAM && algo != SDP_ALGO_PIPE) return 0;
   if (a->warps_per_cta != 0 || (a->ring != 0 && a->ring != 16)) return 0;
   return split_tmem_adj_warps(a->n, a->Q, a->S, num_sms());
@@ -259,26 +247,27 @@ int auto_algo_no_pipe(const sdp_split_args* a) {
   return SDP_ALGO_DEQUE;
 }
 
-bool pipe_ok(const sdp_split_args* a) {
+bool pipe_ok(const sdp_split_args* a, bool host) {
   if (!pipe_supported(a->n, a->Q)) return false;
-  if (a->n > 0 && a->S > 0 && !is_host_ptr(a->demands) &&
+  if (a->n > 0 && a->S > 0 && !host &&
       (reinterpret_cast<uintptr_t>(a->demands) & 15) != 0)
     return false;
   return true;
 }
 
-int resolve_algo(const sdp_split_args* a) {
+// host: the demands are page-locked host memory (demands_of)
+int resolve_algo(const sdp_split_args* a, bool host) {
   int algo = a->algo;
   if (algo != SDP_ALGO_AUTO) return algo;
-  if (a->warps_per_cta == 0 && (a->ring == 0 || a->ring == 16) && pipe_ok(a)) return SDP_ALGO_PIPE;
+  if (a->warps_per_cta == 0 && (a->ring == 0 || a->ring == 16) && pipe_ok(a, host)) return SDP_ALGO_PIPE;
   return auto_algo_no_pipe(a);
 }
 
-SplitWs carve_split(const sdp_split_args* a, void* base, bool backward) {
+SplitWs carve_split(const sdp_split_args* a, void* base, bool backward, bool host) {
   SplitWs w{};
   Carver c{static_cast<unsigned char*>(base)};
   const int n = a->n;
-  const int algo = resolve_algo(a);
+  const int algo = resolve_algo(a, host);
   w.prep.rec = c.take<StepRec>((size_t)n);
   w.prep.cols = c.take<uint16_t>((size_t)n);
   w.prep.Dn = c.take<double>(1);
@@ -297,19 +286,19 @@ SplitWs carve_split(const sdp_split_args* a, void* base, bool backward) {
   w.kscratch = c.take<float>((size_t)(n + 1) * w.nslots);
   w.pscratch = backward ? c.take<int32_t>((size_t)n * w.nslots) : nullptr;
   w.hist = backward ? c.take<unsigned long long>(2 * (size_t)n + 1) : nullptr;
-  w.dscratch = (backward && adjoint_tmem_warps(a) > 0)
+  w.dscratch = (backward && adjoint_tmem_warps(a, host) > 0)
                    ? c.take<uint32_t>(split_tmem_adj_scratch_bytes(n, a->Q, num_sms()) / 4)
                    : nullptr;
   w.qt = nullptr;
   w.tflags = nullptr;
   if (algo == SDP_ALGO_PIPE && !backward && n > 0) {
-    const int64_t rows = (n > 0 && is_host_ptr(a->demands))
+    const int64_t rows = host
                              ? (a->S < kHostChunkRows ? a->S : kHostChunkRows)
                              : a->S;
     w.qt = c.take<unsigned char>(pipe_ring_bytes(n, a->Q, rows, 1, false));
   }
   if (algo == SDP_ALGO_STREAM && !backward && n > 0) {
-    const int64_t rows = (n > 0 && is_host_ptr(a->demands))
+    const int64_t rows = host
                              ? (a->S < kHostChunkRows ? a->S : kHostChunkRows)
                              : a->S;
     w.qt = c.take<unsigned char>(stream_qt_bytes(n, a->Q, rows));
@@ -317,7 +306,7 @@ SplitWs carve_split(const sdp_split_args* a, void* base, bool backward) {
   }
   w.stage[0] = w.stage[1] = nullptr;
   w.stage_rows = 0;
-  if (!backward && n > 0 && a->S > 0 && is_host_ptr(a->demands)) {
+  if (!backward && n > 0 && a->S > 0 && host) {
     w.stage_rows = a->S < kHostChunkRows ? a->S : kHostChunkRows;
     w.stage[0] = c.take<int32_t>((size_t)w.stage_rows * n);
     w.stage[1] = c.take<int32_t>((size_t)w.stage_rows * n);
@@ -326,7 +315,7 @@ SplitWs carve_split(const sdp_split_args* a, void* base, bool backward) {
   return w;
 }
 
-int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
+int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status, bool host,
                    unsigned long long* hist, cudaStream_t st, bool hist_and_cost = false);
 
 // Copy stream and events of the host-demand pipeline, made once per device on
@@ -382,7 +371,7 @@ int run_split_host_chunks(const sdp_split_args* a, const SplitWs& w, uint32_t* s
     c.cost_out = a->cost_out + s0;
     if (a->pred_out)
       c.pred_out = static_cast<unsigned char*>(a->pred_out) + (size_t)s0 * n * pbytes;
-    rc = run_split_core(&c, w, status, nullptr, st);
+    rc = run_split_core(&c, w, status, false, nullptr, st);
     if (rc) return rc;
     e = cudaEventRecord(hp.done[b], st);
     if (e != cudaSuccess) return cuda_fail(e, "host pipeline record");
@@ -390,8 +379,10 @@ int run_split_host_chunks(const sdp_split_args* a, const SplitWs& w, uint32_t* s
   return SDP_OK;
 }
 
-int check_split(const sdp_split_args* a, bool need_cost) {
+// *dem: where a->demands lie
+int check_split(const sdp_split_args* a, bool need_cost, Demands* dem) {
   if (!a) return fail(SDP_ERR_INVALID_ARG, "args is NULL");
+  *dem = demands_of(a->demands);
   if (a->n < 0) return fail(SDP_ERR_INVALID_ARG, "n = %d < 0", a->n);
   if (a->Q <= 0) return fail(SDP_ERR_INVALID_ARG, "Q = %d <= 0", a->Q);
   if (a->S < 0) return fail(SDP_ERR_INVALID_ARG, "S = %lld < 0", (long long)a->S);
@@ -400,7 +391,7 @@ int check_split(const sdp_split_args* a, bool need_cost) {
     return fail(SDP_ERR_INVALID_ARG, "unknown algo %d", a->algo);
   if (a->algo == SDP_ALGO_PIPE && !pipe_supported(a->n, a->Q))
     return fail(SDP_ERR_UNSUPPORTED, "PIPE needs 1 <= n <= %d and Q <= 32767", kPipeMaxN);
-  if (a->algo == SDP_ALGO_PIPE && a->n > 0 && a->S > 0 && !is_host_ptr(a->demands) &&
+  if (a->algo == SDP_ALGO_PIPE && a->n > 0 && a->S > 0 && !dem->host &&
       (reinterpret_cast<uintptr_t>(a->demands) & 15))
     return fail(SDP_ERR_UNSUPPORTED, "PIPE needs 16-byte aligned demands");
   if (a->algo == SDP_ALGO_DEQUE && !deque_supported(a->n, a->Q))
@@ -430,7 +421,7 @@ int check_split(const sdp_split_args* a, bool need_cost) {
       return fail(SDP_ERR_INVALID_ARG, "coords must be a device pointer");
     if (a->dist && !is_device_ptr(a->dist))
       return fail(SDP_ERR_INVALID_ARG, "dist must be a device pointer");
-    if (!device_readable(a->demands))
+    if (!dem->ptr)
       return fail(SDP_ERR_INVALID_ARG,
                   "demands must be device memory or page-locked host memory mapped for the device");
   }
@@ -464,9 +455,9 @@ int check_ws(void* ws, size_t have, size_t need) {
 // flagged (one warp each where its rows fit split_rescue.cu's shared memory;
 // else the plain kernel over the flagged list), or runs the PLAIN kernel over
 // all S.  With route counts (hist) costs are written only if hist_and_cost.
-int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
+int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status, bool host,
                    unsigned long long* hist, cudaStream_t st, bool hist_and_cost) {
-  int algo = resolve_algo(a);
+  int algo = resolve_algo(a, host);
   if ((algo == SDP_ALGO_STREAM || algo == SDP_ALGO_PIPE) && hist)
     algo = SDP_ALGO_DEQUE;  // the fused adjoint is DEQUE's
   const int sms = num_sms();
@@ -510,7 +501,7 @@ int run_split_core(const sdp_split_args* a, const SplitWs& w, uint32_t* status,
     prof_end(st);
     if (e) return cuda_fail((cudaError_t)e, "split_pipe launch");
   }
-  const int adj_warps = (hist && w.dscratch) ? adjoint_tmem_warps(a) : 0;
+  const int adj_warps = (hist && w.dscratch) ? adjoint_tmem_warps(a, host) : 0;
   if (algo == SDP_ALGO_DEQUE && adj_warps > 0) {
     SplitDequeArgs d{};
     d.n = a->n; d.Q = a->Q; d.S = a->S;
@@ -680,29 +671,30 @@ int sdp_device_status(int clear, uint32_t* flags_out) {
 
 size_t sdp_split_workspace_bytes(const sdp_split_args* a) {
   if (!a || a->n < 0 || a->S < 0) return 0;
-  return carve_split(a, nullptr, false).bytes;
+  return carve_split(a, nullptr, false, demands_of(a->demands).host).bytes;
 }
 
 size_t sdp_split_backward_workspace_bytes(const sdp_split_args* a) {
   if (!a || a->n < 0 || a->S < 0) return 0;
-  return carve_split(a, nullptr, true).bytes;
+  return carve_split(a, nullptr, true, demands_of(a->demands).host).bytes;
 }
 
 int sdp_split_eval(const sdp_split_args* args, void* stream) {
-  int rc = check_split(args, true);
+  Demands dem;
+  int rc = check_split(args, true, &dem);
   if (rc) return rc;
-  const sdp_split_args rd = with_readable_demands(args);
-  const sdp_split_args* a = &rd;
+  sdp_split_args readable = *args;
+  readable.demands = dem.ptr;
+  const sdp_split_args* a = &readable;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const SplitWs need = carve_split(a, nullptr, false);
-  rc = check_ws(a->workspace, a->workspace_bytes, need.bytes);
+  const SplitWs w = carve_split(a, a->workspace, false, dem.host);
+  rc = check_ws(a->workspace, a->workspace_bytes, w.bytes);
   if (rc) return rc;
   uint32_t* status;
   rc = status_ptr(&status);
   if (rc) return rc;
   rc = fault_call();
   if (rc) return rc;
-  const SplitWs w = carve_split(a, a->workspace, false);
   if (a->S > 0 && a->n == 0) {
     cudaError_t e = cudaMemsetAsync(a->cost_out, 0, sizeof(float) * a->S, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(mean_counter(w.mean_partial), 0, sizeof(uint32_t), st);
@@ -715,7 +707,7 @@ int sdp_split_eval(const sdp_split_args* args, void* stream) {
     // host demands: copied chunk by chunk (from the caller's host address)
     // behind the evaluation of the previous chunk
     rc = w.stage_rows > 0 ? run_split_host_chunks(args, w, status, st)
-                          : run_split_core(a, w, status, nullptr, st);
+                          : run_split_core(a, w, status, dem.host, nullptr, st);
     if (rc) return rc;
   }
   if (a->mean_out) {
@@ -824,7 +816,8 @@ FleetWs carve_fleet(const sdp_split_args* a, int K, bool routes, void* base) {
 }
 
 int check_fleet(const sdp_split_args* a, int32_t K) {
-  int rc = check_split(a, true);
+  Demands dem;
+  int rc = check_split(a, true, &dem);
   if (rc) return rc;
   if (K < 1 || K > kFleetMaxK) return fail(SDP_ERR_UNSUPPORTED, "max_routes = %d outside 1..%d", K, kFleetMaxK);
   if (a->n > 16384) return fail(SDP_ERR_UNSUPPORTED, "fleet-limited Split needs n <= 16384");
@@ -858,15 +851,14 @@ int sdp_split_fleet_eval(const sdp_split_args* a, int32_t max_routes, int32_t* n
     return fail(SDP_ERR_INVALID_ARG, "route_out must be a device pointer");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool routes = route_out != nullptr && a->n > 0;
-  const FleetWs need = carve_fleet(a, max_routes, routes, nullptr);
-  rc = check_ws(a->workspace, a->workspace_bytes, need.bytes);
+  const FleetWs w = carve_fleet(a, max_routes, routes, a->workspace);
+  rc = check_ws(a->workspace, a->workspace_bytes, w.bytes);
   if (rc) return rc;
   uint32_t* status;
   rc = status_ptr(&status);
   if (rc) return rc;
   rc = fault_call();
   if (rc) return rc;
-  const FleetWs w = carve_fleet(a, max_routes, routes, a->workspace);
   if (a->S > 0 && a->n == 0) {
     cudaError_t e = cudaMemsetAsync(a->cost_out, 0, sizeof(float) * a->S, st);
     if (e == cudaSuccess && nroutes_out) e = cudaMemsetAsync(nroutes_out, 0, sizeof(int32_t) * a->S, st);
@@ -913,20 +905,21 @@ int sdp_split_fleet_eval(const sdp_split_args* a, int32_t max_routes, int32_t* n
 
 int sdp_split_count_arcs(const sdp_split_args* args, int64_t* arcs_out, uint64_t* total_out,
                          void* stream) {
-  int rc = check_split(args, false);
+  Demands dem;
+  int rc = check_split(args, false, &dem);
   if (rc) return rc;
-  const sdp_split_args rd = with_readable_demands(args);
-  const sdp_split_args* a = &rd;
+  sdp_split_args readable = *args;
+  readable.demands = dem.ptr;
+  const sdp_split_args* a = &readable;
   if (arcs_out && !is_device_ptr(arcs_out)) return fail(SDP_ERR_INVALID_ARG, "arcs_out must be a device pointer");
   if (total_out && !is_device_ptr(total_out)) return fail(SDP_ERR_INVALID_ARG, "total_out must be a device pointer");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const SplitWs need = carve_split(a, nullptr, false);
-  rc = check_ws(a->workspace, a->workspace_bytes, need.bytes);
+  const SplitWs w = carve_split(a, a->workspace, false, dem.host);
+  rc = check_ws(a->workspace, a->workspace_bytes, w.bytes);
   if (rc) return rc;
   uint32_t* status;
   rc = status_ptr(&status);
   if (rc) return rc;
-  const SplitWs w = carve_split(a, a->workspace, false);
   if (total_out) {
     cudaError_t e = cudaMemsetAsync(total_out, 0, sizeof(uint64_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "memset total");
@@ -949,10 +942,12 @@ int sdp_split_count_arcs(const sdp_split_args* args, int64_t* arcs_out, uint64_t
 
 int sdp_split_backward(const sdp_split_args* args, const void* pred, const float* grad_mean,
                        float* grad_dist, int64_t* route_hist_out, void* stream) {
-  int rc = check_split(args, false);
+  Demands dem;
+  int rc = check_split(args, false, &dem);
   if (rc) return rc;
-  const sdp_split_args rd = with_readable_demands(args);
-  const sdp_split_args* fwd = &rd;
+  sdp_split_args readable = *args;
+  readable.demands = dem.ptr;
+  const sdp_split_args* fwd = &readable;
   if (!fwd->dist) return fail(SDP_ERR_UNSUPPORTED, "the adjoint is taken with respect to dist: set dist, not coords");
   if (fwd->capacity_mode != SDP_CAPACITY_HARD)
     return fail(SDP_ERR_UNSUPPORTED, "the adjoint takes the hard capacity only");
@@ -964,20 +959,19 @@ int sdp_split_backward(const sdp_split_args* args, const void* pred, const float
   if (pred && fwd->pred_dtype != SDP_PRED_U16 && fwd->pred_dtype != SDP_PRED_I32)
     return fail(SDP_ERR_INVALID_ARG, "pred_dtype must be SDP_PRED_U16 or SDP_PRED_I32");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const SplitWs need = carve_split(fwd, nullptr, true);
-  rc = check_ws(fwd->workspace, fwd->workspace_bytes, need.bytes);
+  const SplitWs w = carve_split(fwd, fwd->workspace, true, dem.host);
+  rc = check_ws(fwd->workspace, fwd->workspace_bytes, w.bytes);
   if (rc) return rc;
   uint32_t* status;
   rc = status_ptr(&status);
   if (rc) return rc;
   rc = fault_call();
   if (rc) return rc;
-  const SplitWs w = carve_split(fwd, fwd->workspace, true);
   const int n = fwd->n;
   if (n > 0 && fwd->S > 0 && !pred) {
     launch_tour_prep(fwd->tour, n, fwd->coords, fwd->dist, w.prep, status,
                      {w.fb_count, w.counter, nullptr, w.hist}, st);
-    rc = run_split_core(fwd, w, status, w.hist, st);
+    rc = run_split_core(fwd, w, status, dem.host, w.hist, st);
     if (rc) return rc;
   } else {
     const cudaError_t e = cudaMemsetAsync(w.hist, 0, sizeof(unsigned long long) * (2 * (size_t)n + 1), st);
@@ -991,33 +985,37 @@ int sdp_split_backward(const sdp_split_args* args, const void* pred, const float
 }
 
 // ------------------------------------------- costs and route counts together
+static bool routes_fused(const sdp_split_args* a, const Demands& dem) {
+  return a->n > 0 && a->S > 0 && a->Q > 0 && a->capacity_mode == SDP_CAPACITY_HARD && !dem.host &&
+         adjoint_tmem_warps(a, false) > 0;
+}
+
 size_t sdp_split_routes_workspace_bytes(const sdp_split_args* a) {
-  if (!a || a->n < 1 || a->S < 1 || a->Q <= 0 || a->capacity_mode != SDP_CAPACITY_HARD ||
-      is_host_ptr(a->demands) || adjoint_tmem_warps(a) < 1)
-    return 0;
-  return carve_split(a, nullptr, true).bytes + (a->cost_out ? 0 : sizeof(float) * (size_t)a->S);
+  if (!a || !routes_fused(a, demands_of(a->demands))) return 0;
+  return carve_split(a, nullptr, true, false).bytes + (a->cost_out ? 0 : sizeof(float) * (size_t)a->S);
 }
 
 int sdp_split_eval_routes(const sdp_split_args* args, uint64_t* routes_out, void* stream) {
-  int rc = check_split(args, false);
+  Demands dem;
+  int rc = check_split(args, false, &dem);
   if (rc) return rc;
   if (args->cost_out && !is_device_ptr(args->cost_out))
     return fail(SDP_ERR_INVALID_ARG, "cost_out must be a device pointer");
   if (!is_device_ptr(routes_out)) return fail(SDP_ERR_INVALID_ARG, "routes_out must be a device pointer");
   if (args->pred_out)
     return fail(SDP_ERR_INVALID_ARG, "sdp_split_eval_routes returns route counts, not pred_out");
-  const size_t need = sdp_split_routes_workspace_bytes(args);
-  if (need == 0)
+  if (!routes_fused(args, dem))
     return fail(SDP_ERR_UNSUPPORTED, "this shape has no kernel that returns costs and route counts together");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  rc = check_ws(args->workspace, args->workspace_bytes, need);
+  const SplitWs w = carve_split(args, args->workspace, true, false);
+  rc = check_ws(args->workspace, args->workspace_bytes,
+                w.bytes + (args->cost_out ? 0 : sizeof(float) * (size_t)args->S));
   if (rc) return rc;
   uint32_t* status;
   rc = status_ptr(&status);
   if (rc) return rc;
   rc = fault_call();
   if (rc) return rc;
-  const SplitWs w = carve_split(args, args->workspace, true);
   sdp_split_args with_cost = *args;
   const sdp_split_args* a = &with_cost;
   if (!a->cost_out)
@@ -1027,7 +1025,7 @@ int sdp_split_eval_routes(const sdp_split_args* args, uint64_t* routes_out, void
                    {w.fb_count, w.counter, mean_counter(w.mean_partial), routes}, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "tour_prep launch");
-  rc = run_split_core(a, w, status, routes, st, true);
+  rc = run_split_core(a, w, status, false, routes, st, true);
   if (rc) return rc;
   if (a->mean_out) {
     launch_mean(a->cost_out, a->S, w.mean_partial, a->mean_out, st);
