@@ -30,15 +30,19 @@
 //
 // What bounds it: the fixed latencies of a cell's dependent operations with
 // 8 warps per SM (14 bytes of shared memory per scenario-day).  At T = 60,
-// U = 200, mean consumption 8, S = 10^6: 219 warp instructions per day and 32
-// scenarios against about 2,100 for the lane kernel; 0.71 ms, the lane kernel
-// 5.20 ms.  Four routes: 2.3 ms against 9.9.  One chain at a time with loops
-// of each lane's own length took 1.14 ms (the decisions recorded in every
-// cell); two chains the same.
+// U = 200, mean consumption 8, S = 10^6: 230 warp instructions per day and 32
+// scenarios against about 2,100 for the lane kernel; 0.65 ms, the lane kernel
+// 5.20 ms.  Four routes: 2.22 ms against 9.9.  Loading a day's record while
+// the day above runs gave 5% of that (routes 1%), the L2 prefetch of the next
+// tile's rows 4% (3%).  11 warps per SM (16-bit prefix sums, decisions as bits)
+// took 263 instructions a day and the same time.  One chain at a time with
+// loops of each lane's own length took 1.14 ms (the decisions recorded in
+// every cell); two chains the same.
 //
 #include <math.h>
 #include <math_constants.h>
 
+#include "async_copy.cuh"
 #include "dependent.cuh"
 #include "sdp_internal.cuh"
 
@@ -120,6 +124,18 @@ __global__ void __launch_bounds__(kChainMaxWarps * 32, 1) reinsert_chain_kernel(
        tile += (int64_t)gridDim.x * nwarps) {
     const int64_t s0 = tile * 32;
     const bool live = lane < a.S - s0;
+    // the warp's next rows on their way to L2 meanwhile
+    const int64_t next = s0 + 32 * (int64_t)gridDim.x * nwarps;
+    if (lane == 0 && next < a.S) {
+      const int64_t rows = imin64(32, a.S - next);
+      auto ahead = [&](const int32_t* p, int64_t row) {
+        p += next * row;
+        if ((reinterpret_cast<uintptr_t>(p) & 15) == 0 && rows * row >= 4)
+          bulk_prefetch_l2(p, (uint32_t)(rows * row * 4) & ~15u);
+      };
+      ahead(a.cons, T);
+      if (RK > 0) ahead(a.route_cap, (int64_t)T * K);
+    }
     // a lane without a scenario follows the tile's first
     const int32_t* crow = a.cons + (s0 + (live ? lane : 0)) * T;
     const int32_t* caprow = RK > 0 ? a.route_cap + (s0 + (live ? lane : 0)) * (int64_t)T * K : nullptr;
@@ -267,16 +283,21 @@ __global__ void __launch_bounds__(kChainMaxWarps * 32, 1) reinsert_chain_kernel(
           for (int j = 0; j < kChains; ++j)
             nd[j] = left(Flag<SLOW>{}, A[j], __fsub_rn(A[j], Pz), -0.f, z, zhi);
         }
+        // the next day's record is loaded while this day's cells run
         int s = zhi - 1;
+        float2 v = bp[max(s, 0) * 32];
 #pragma unroll 1
         for (; s >= zlo; --s) {
-          const float2 v = bp[s * 32];
+          const float2 vn = bp[max(s - 1, 0) * 32];
           cells(Flag<true>{}, s, v, zs[s * 32], A, nd);
+          v = vn;
         }
         if (!SLOW) {
-#pragma unroll 2
+#pragma unroll 4
           for (; s > t; --s) {
-            cells(Flag<false>{}, s, bp[s * 32], 0.f, A, nd);
+            const float2 vn = bp[max(s - 1, 0) * 32];
+            cells(Flag<false>{}, s, v, 0.f, A, nd);
+            v = vn;
           }
         }
         // days t .. t - 3: each chain comes down to its day, which gives that
