@@ -159,6 +159,7 @@ struct BatchPrepArgs {
   unsigned long long* counter;  // reset to 0 by the prep kernel
   uint32_t* fb_count;           // reset to 0 by the prep kernel
   uint32_t* status;
+  int32_t* prefix;              // [B] leading records equal to tour 0's, or NULL (tours of one length)
 };
 void launch_batch_prep(const BatchPrepArgs& a, int B, cudaStream_t st);
 void launch_batch_means(const float* costs, int B, int64_t S, double* means, cudaStream_t st);
@@ -310,6 +311,7 @@ struct PipeArgs {
   uint32_t* status;
   uint64_t wait_ns;            // a bounded wait gives up after this
   int stall;                   // fault injection (tests): producers publish no tile
+  const int32_t* prefix;       // split_shared: [B] leading records equal to tour 0's
   int after_prep;              // the stream's previous operation is the tour preparation
 };
 bool pipe_supported(int n, int Q);

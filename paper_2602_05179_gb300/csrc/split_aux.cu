@@ -355,7 +355,8 @@ namespace sdp {
 
 // ------------------------------------------------------------ batched Split
 // Tour prep for every tour of a batch: one CTA per tour, same arithmetic as
-// tour_prep_kernel.
+// tour_prep_kernel.  With a.prefix, tour 0's records are made alongside, to
+// count the leading ones that the tour shares with it.
 __global__ void __launch_bounds__(256) batch_prep_kernel(BatchPrepArgs a) {
   __shared__ double red[256];
   const int b = blockIdx.x;
@@ -367,30 +368,51 @@ __global__ void __launch_bounds__(256) batch_prep_kernel(BatchPrepArgs a) {
     *a.counter = 0ull;
     *a.fb_count = 0u;
   }
+  __shared__ int same;
+  if (threadIdx.x == 0) same = n;
+  __syncthreads();
   double acc = 0.0;
   bool bad = false;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    int si = __ldg(tour + i);
+  int differs = n;
+  // record i of a tour, and its arc from the position before
+  auto record = [&](const int32_t* t, const float* xy, int i, float* arc) -> StepRec {
+    int si = __ldg(t + i);
     if (si < 1 || si > n) { bad = true; si = 1; }
-    const float c0 = travel(coords, nullptr, n, 0, si);
-    const float ce = travel(coords, nullptr, n, si, 0);
+    const float c0 = travel(xy, nullptr, n, 0, si);
+    const float ce = travel(xy, nullptr, n, si, 0);
     float e = 0.f;
     if (i > 0) {
-      int sp = __ldg(tour + i - 1);
+      int sp = __ldg(t + i - 1);
       if (sp < 1 || sp > n) sp = 1;
-      e = travel(coords, nullptr, n, sp, si);
-      acc += (double)e;
+      e = travel(xy, nullptr, n, sp, si);
     }
+    *arc = e;
     StepRec r;
     r.col = (uint32_t)(si - 1);
     r.a = __fsub_rn(c0, e);
     r.ce = ce;
     r.pad = 0u;
+    return r;
+  };
+  const int32_t* tour0 = a.tours + a.tour_off[0];
+  const float* coords0 = a.coords + 2 * a.coord_off[0];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    float e;
+    const StepRec r = record(tour, coords, i, &e);
+    if (i > 0) acc += (double)e;
     rec[i] = r;
+    if (a.prefix && b > 0 && differs == n) {
+      const StepRec r0 = record(tour0, coords0, i, &e);
+      if (r.col != r0.col || __float_as_uint(r.a) != __float_as_uint(r0.a) ||
+          __float_as_uint(r.ce) != __float_as_uint(r0.ce))
+        differs = i;
+    }
   }
   if (bad) atomicOr(a.status, SDP_FLAG_DEVICE_CHECK);
+  if (differs < n) atomicMin(&same, differs);
   red[threadIdx.x] = acc;
   __syncthreads();
+  if (a.prefix && threadIdx.x == 0) a.prefix[b] = same;
   for (int w = blockDim.x / 2; w > 0; w >>= 1) {
     if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
     __syncthreads();

@@ -50,6 +50,7 @@ struct sdp_plan {
   unsigned long long* d_total = nullptr;
   unsigned char* d_qt = nullptr;  // row slots of the streaming kernel, or NULL
   unsigned char* d_pq = nullptr;  // slot ring of the pipelined kernel, or NULL
+  int32_t* d_prefix = nullptr;    // shared: [B] leading records equal to tour 0's
   bool shared = false;            // one length and one demand array for every tour
   // caller's arrays
   const int32_t* tours = nullptr;
@@ -101,6 +102,7 @@ BatchPrepArgs prep_args(const sdp_plan* p, uint32_t* status) {
   a.counter = p->d_counter;
   a.fb_count = p->d_fb_count;
   a.status = status;
+  a.prefix = p->d_prefix;
   return a;
 }
 
@@ -164,6 +166,7 @@ int enqueue(sdp_plan* p, cudaStream_t st, uint32_t* status, bool with_events) {
     pa.qt = p->d_pq; pa.stride = pipe_row_stride(p->n_max, p->Q); pa.counter = p->d_counter;
     pa.n_max = p->n_max;
     pa.fb_count = p->d_fb_count; pa.fb_list = p->d_fb_list; pa.status = status;
+    pa.prefix = p->d_prefix;
     e = p->shared ? launch_split_shared(pa, st) : launch_split_pipe(pa, st);
   } else if (p->warps < 0) {
     BatchStreamArgs sa{};
@@ -237,7 +240,7 @@ void sdp_plan_destroy(sdp_plan* p) {
   cudaFree(p->d_dem_off); cudaFree(p->d_rec_off); cudaFree(p->d_order);
   cudaFree(p->d_rec); cudaFree(p->d_Dn); cudaFree(p->d_counter); cudaFree(p->d_fb_count);
   cudaFree(p->d_fb_list); cudaFree(p->d_kscratch); cudaFree(p->d_total); cudaFree(p->d_qt);
-  cudaFree(p->d_pq);
+  cudaFree(p->d_pq); cudaFree(p->d_prefix);
   if (p->ev0) cudaEventDestroy(p->ev0);
   if (p->ev1) cudaEventDestroy(p->ev1);
   cudaSetDevice(prev);
@@ -306,6 +309,7 @@ int sdp_split_plan_create(const sdp_split_batch_desc* d, sdp_plan** out) {
   p->shared = p->d_pq != nullptr && shared_supported(p->n_max, p->Q, p->B);
   for (int b = 1; p->shared && b < d->B; ++b)
     p->shared = d->n_host[b] == d->n_host[0] && d->dem_off_host[b] == d->dem_off_host[0];
+  if (p->shared) chk(alloc_copy<int32_t>(&p->d_prefix, nullptr, d->B));
   if (e == cudaSuccess) e = cudaEventCreate(&p->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&p->ev1);
   if (e != cudaSuccess) {
