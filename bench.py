@@ -542,8 +542,10 @@ def op_reinsert(c, out):
     rel = 2.0 * (rs.U + 1) * rs.T * rs.S
     line = {"value": rel / (ms / 1e3), "unit": "relaxations/s",
             "scenarios_per_s": rs.S / (ms / 1e3), "ms_per_step": ms, "kernel_ms": kms,
-            "kernel": "reinsert_lane_kernel (one scenario per lane)",
-            "roofline": c.alu_roof(2 * rel, kms),
+            "kernel": "reinsert_chain_kernel (reachable states, one scenario per lane)",
+            # value counts the states of the whole recursion; the roofline credits
+            # the at most t + 1 of them that day t can start in
+            "roofline": c.alu_roof(2 * rs.S * sum(min(t + 1, rs.U + 1) for t in range(rs.T)), kms),
             "vs_plain": {"kernel": "reinsert_kernel (one scenario per warp)",
                          "ms_per_step": wms, "kernel_ms": wkms, "speedup": wkms / kms,
                          "values_bit_identical": bool(torch.equal(r["value"], rw["value"])),
@@ -581,8 +583,8 @@ def op_routes(c, out):
     rel = float(rr.U + 1) * rr.T * (K + 1) * rr.S  # (state, action) pairs
     line = {"value": rel / (ms / 1e3), "unit": "relaxations/s",
             "scenarios_per_s": rr.S / (ms / 1e3), "ms_per_step": ms, "kernel_ms": kms,
-            "kernel": "reinsert_lane_kernel (route options, one scenario per lane)",
-            "roofline": c.alu_roof(2 * rel, kms),
+            "kernel": "reinsert_chain_kernel (route options, reachable states, one scenario per lane)",
+            "roofline": c.alu_roof(2 * rr.S * (K + 1) * sum(min(t + 1, rr.U + 1) for t in range(rr.T)), kms),
             "vs_warp": {"kernel": "reinsert_routes_kernel (one scenario per warp)", "ms_per_step": wms,
                         "kernel_ms": wkms, "speedup": wkms / kms, "bit_identical": same}}
     if c.checks:
@@ -734,11 +736,12 @@ def op_fleet(c, out):
     same = all(bool(torch.equal(r[k][:Sp], rp[k])) for k in ("cost", "nroutes", "route"))
     fin = torch.isfinite(r["cost"])
     line = {"value": S / (ms / 1e3), "unit": "scenarios/s", "ms_per_step": ms, "kernel_ms": kms,
-            "kernel": "split_fleet_kernel (one warp per scenario, route counts across lanes)",
+            "kernel": "split_fleet_band_kernel (one warp per scenario, positions across lanes)",
             "max_routes": K, "feasible_frac": float(fin.float().mean()),
             "flagged_recomputed": fell_back,
-            "recompute": "scenarios whose deques outgrow the ring: split_fleet_rescue_kernel, one warp "
-                         "per scenario, inside ms_per_step (the roofline is the main kernel's)",
+            "recompute": "scenarios with windows of more than 32 positions: the same kernel in wider "
+                         "blocks, inside ms_per_step",
+            # of the whole recursion; the kernel evaluates the band that K routes leave
             "layer_relaxations_per_s": rel / (kms / 1e3),
             "roofline": c.alu_roof(2 * rel, kms),
             "vs_plain": {"path": "one thread per scenario, every feasible p of every layer",

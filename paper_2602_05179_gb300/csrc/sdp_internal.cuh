@@ -234,7 +234,7 @@ struct StreamArgs {
   float* cost;
   void* pred;               // nullable
   int pred_dtype;
-  uint32_t* fb_list;        // [S] scenarios recomputed by the plain kernel
+  uint32_t* fb_list;        // [S] ids of the flagged scenarios
   uint32_t* fb_count;
   uint32_t* status;
   int ctas_per_sm;          // CTAs per SM (0 = 1)
@@ -306,7 +306,7 @@ struct PipeArgs {
   int64_t stride;              // bytes per slot row (pipe_row_stride of the longest tour)
   unsigned long long* counter; // group queue, zero at launch
   uint32_t* fb_count;
-  uint32_t* fb_list1;          // one tour: [S] scenario ids for the plain kernel
+  uint32_t* fb_list1;          // one tour: [S] ids of the flagged scenarios
   unsigned long long* fb_list; // batched: [B*S] global ids b*S+s
   uint32_t* status;
   uint64_t wait_ns;            // a bounded wait gives up after this

@@ -18,9 +18,8 @@
 //   - the front is the argmin (kept in registers).
 // The deque is a ring of RING entries per lane in shared memory, laid out
 // [entry][lane] so every access is bank-conflict free.  A scenario whose
-// deque outgrows the ring is flagged and recomputed: by one warp
-// (split_rescue.cu) for hard capacity, by the plain kernel for soft capacity
-// and the adjoint.
+// deque outgrows the ring is flagged and recomputed by one warp
+// (split_rescue.cu).
 //
 // Demand staging (two variants of the same DP).
 //   Shared memory: the tile's rows are contiguous in HBM (row-major [S, n]);
