@@ -420,9 +420,11 @@ __global__ void __launch_bounds__(kSWarps * 32, 1) split_shared_kernel(PipeArgs 
   }
 }
 
+// dynamic shared memory of a CTA: 227 KB less the kernel's own variables
+constexpr size_t kSSmemMax = 227 * 1024 - 256;
 size_t shared_smem(int n, int Q) {
   return (size_t)(kSWarps + 1) * kSRingBytes + (size_t)kSWarps * kSRecs * 16 +
-         (size_t)n * 32 * (Q <= 254 ? 1 : 2);
+         (size_t)n * 32 * (Q <= 254 ? 1 : 2) + 16;
 }
 
 template <typename QT>
@@ -430,14 +432,14 @@ int launch_s(const PipeArgs& a, int grid, cudaStream_t st) {
   auto k = split_shared_kernel<QT>;
   // tour 0's states: as many as fit, every 8 positions at best (the last one
   // before position n)
-  const size_t tiles = shared_smem(a.n_max, a.Q) + 16;
-  const int fit = tiles < 227 * 1024 ? (int)((227 * 1024 - tiles) / kSStateBytes) : 0;
+  const size_t tiles = shared_smem(a.n_max, a.Q);
+  const int fit = tiles < kSSmemMax ? (int)((kSSmemMax - tiles) / kSStateBytes) : 0;
   int step = 0, count = 0;
   if (a.prefix && fit > 0 && a.n_max > 8) {
     step = (((a.n_max - 1) / 8 + fit - 1) / fit) * 8;
     count = std::min(fit, (a.n_max - 1) / step);
   }
-  const size_t smem = std::min<size_t>(227 * 1024, tiles + (size_t)count * kSStateBytes);
+  const size_t smem = tiles + (size_t)count * kSStateBytes;
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
   k<<<grid, kSWarps * 32, smem, st>>>(a, step, count);
@@ -449,7 +451,7 @@ int launch_s(const PipeArgs& a, int grid, cudaStream_t st) {
 // At least two tours per warp, so that a staged tile keeps the warps busy.
 bool shared_supported(int n, int Q, int B) {
   return n >= 1 && n <= 65535 && Q >= 1 && Q <= 32767 && B >= 2 * kSWarps &&
-         shared_smem(n, Q) <= 227 * 1024;
+         shared_smem(n, Q) <= kSSmemMax;
 }
 
 int launch_split_shared(const PipeArgs& a, cudaStream_t st) {

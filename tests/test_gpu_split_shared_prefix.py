@@ -21,6 +21,8 @@ def _cuda(x):
     (100, 64, 240, 20, (-2, 22), False),
     (67, 70, 96, 60, (0, 3), True),
     (600, 100, 70, 400, (1, 30), False),
+    (127, 40, 64, 100, (1, 30), False),      # states that fill the shared memory to within 16 bytes
+    (64, 40, 64, 300, (1, 60), False),
 ])
 def test_prefixes_equal_single(case):
     from paper_2602_05179_gb300 import api
