@@ -399,6 +399,9 @@ __global__ void __launch_bounds__(kSWarps * 32, 1) split_shared_kernel(PipeArgs 
       int from = 0;
       if (resume) {
         if (lane == 0) from = min(a.prefix[b] / snap_step, (int)ld_acquire_shared(&snap_ready));
+        // lane 0's acquire orders its own reads only; the barrier carries the
+        // order to the lanes that read the state with it (a shuffle does not)
+        __syncwarp();
         from = __shfl_sync(kAll, from, 0);
       }
       if (tf) run_tour<QT, true, false>(n, Q, tile, ring, recs, rec, lane, snap, 0, &K, &first_inf, &bad);
