@@ -523,7 +523,7 @@ def _grad_from_routes(tour, S, routes, grad_mean):
     """d mean / d dist (fp32 [n+1, n+1]) times grad_mean from route counts."""
     n = int(tour.numel())
     grad = torch.empty((n + 1, n + 1), dtype=torch.float32, device=tour.device)
-    gm = grad_mean
+    gm = grad_mean.resolve_neg()  # its memory is read: a lazily negated one holds the other sign
     if gm.device != tour.device or gm.dtype not in (torch.float32, torch.float64):
         gm = gm.to(device=tour.device, dtype=torch.float32)
     _check(_load().sdp_split_grad_from_routes(n, S, tour.data_ptr(), routes.data_ptr(), gm.data_ptr(),
