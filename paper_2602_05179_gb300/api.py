@@ -526,7 +526,9 @@ def _grad_from_routes(tour, S, routes, grad_mean):
     gm = grad_mean.resolve_neg()  # its memory is read: a lazily negated one holds the other sign
     if gm.device != tour.device or gm.dtype not in (torch.float32, torch.float64):
         gm = gm.to(device=tour.device, dtype=torch.float32)
-    _check(_load().sdp_split_grad_from_routes(n, S, tour.data_ptr(), routes.data_ptr(), gm.data_ptr(),
+    # a saved-tensor hook may have put other tensors in the place of these two
+    _check(_load().sdp_split_grad_from_routes(n, S, _dev_ptr(tour, "tour", torch.int32),
+                                              _dev_ptr(routes, "routes", torch.int64), gm.data_ptr(),
                                               1 if gm.dtype == torch.float64 else 0, grad.data_ptr(),
                                               _stream(None)))
     return grad

@@ -30,3 +30,26 @@ def test_lazily_negated_gradient(dt):
         gn = api._grad_from_routes(tour, qd.shape[0], api._split_mean_routes(tour, Q, qd, leaf.detach())[1],
                                    torch._neg_view(torch.ones((), dtype=dt, device="cuda")))
     assert torch.equal(gn, -g)
+
+
+@pytest.mark.parametrize("form", ["int64", "strided"])
+@pytest.mark.parametrize("which", ["tour", "routes"])
+def test_unpacked_tensors_of_another_form_are_refused(which, form):
+    """A saved-tensor hook's unpacked tour or route counts are checked as the
+    forward's inputs are."""
+    from paper_2602_05179_gb300 import api
+    leaf, tour, qd, Q = _problem()
+    n = tour.numel()
+
+    def unpack(t):
+        hit = t.dtype == torch.int32 and t.numel() == n if which == "tour" else t.numel() == 2 * n + 1
+        if not hit:
+            return t
+        if form == "int64":
+            return t.to(torch.int64 if which == "tour" else torch.int32)
+        return torch.stack((t, t), 1)[:, 0]
+
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: t, unpack):
+        m = api.SplitMeanCost.apply(leaf, tour, qd, Q)
+        with pytest.raises(ValueError):
+            m.backward()
