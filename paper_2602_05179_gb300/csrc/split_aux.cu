@@ -106,22 +106,32 @@ void launch_count_arcs(int n, int Q, int64_t S, const StepRec* rec,
 }
 
 // ------------------------------------------------------------- FP64 mean
-// Eight values as the pair of floats (their rounded sum, the exact sum of its
-// rounding errors by Knuth's two-sum) and then one FP64 number: exact for
-// values within 2^20 of each other, so the sum of any group is what FP64
-// additions give.  GB300 has few FP64 units (a conversion and an addition per
-// value took 48 us for 1,025 x 10^4 values; 0.25 of each per value here).
+// Eight values as the pair of floats (their rounded sum, the sum of its rounding
+// errors by Knuth's two-sum) and then one FP64 number.  GB300 has few FP64 units
+// (a conversion and an addition per value took 48 us for 1,025 x 10^4 values;
+// 0.25 of each per value here).  The pair is taken only where it is exact:
+// where the largest magnitude M and the least one above zero, m, are at most 19
+// binary exponents apart.  With u the last place of m, all sums and errors are
+// multiples of u; a partial sum is at most 8 M, so the seven errors add up to
+// at most 28 last places of M <= 2^24 u, which a float holds, and the two parts
+// to 46 bits, which a double holds.  Other groups (a spread of 2^20 or more, an
+// infinity, a NaN, a sum beyond the largest float) are added in FP64.
 __device__ __forceinline__ double sum8(const float* v) {
-  float hi = v[0], lo = 0.f;
+  float hi = v[0], lo = 0.f, big = fabsf(v[0]);
+  uint32_t least = 2u * __float_as_uint(v[0]) - 1u;  // magnitudes in order, zero as the last
 #pragma unroll
   for (int k = 1; k < 8; ++k) {
     const float s = __fadd_rn(hi, v[k]);
     const float t = __fsub_rn(s, hi);
     lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(v[k], t)));
     hi = s;
+    big = fmaxf(big, fabsf(v[k]));
+    least = min(least, 2u * __float_as_uint(v[k]) - 1u);
   }
-  if (fabsf(hi) <= 3.0e38f) return (double)hi + (double)lo;
-  double acc = 0.0;  // an infinity, a NaN or an overflow of the float sum
+  // (all zeros: least is the largest word, and the test holds)
+  if (fabsf(hi) <= 3.0e38f && (__float_as_uint(big) >> 23) <= (least >> 24) + 19u)
+    return (double)hi + (double)lo;
+  double acc = 0.0;
 #pragma unroll
   for (int k = 0; k < 8; ++k) acc += (double)v[k];
   return acc;
