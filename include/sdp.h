@@ -541,7 +541,12 @@ typedef struct sdp_reinsert_args {
 } sdp_reinsert_args;
 
 size_t sdp_reinsert_args_size(void);
+/* sdp_reinsert_workspace_bytes: enough for these arguments with and without
+ * value0_out; sdp_reinsert_call_bytes: what the call with exactly these
+ * arguments needs (4 KB where AUTO takes the reachable-state kernel, which
+ * keeps no decision bits in the workspace). */
 size_t sdp_reinsert_workspace_bytes(const sdp_reinsert_args* a);
+size_t sdp_reinsert_call_bytes(const sdp_reinsert_args* a);
 int sdp_reinsert_eval(const sdp_reinsert_args* a, void* stream);
 
 #ifdef __cplusplus

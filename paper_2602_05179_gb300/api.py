@@ -115,6 +115,7 @@ def _load_once():
             "sdp_split_eval_routes": ([P, P, P], i32),
             "sdp_split_grad_from_routes": ([i32, i64, P, P, P, i32, P, P], i32),
             "sdp_reinsert_workspace_bytes": ([P], sz),
+            "sdp_reinsert_call_bytes": ([P], sz),
             "sdp_reinsert_eval": ([P, P], i32),
             "sdp_set_profile_events": ([P, P], i32),
             "sdp_last_launch": ([P, P], i32),
@@ -569,7 +570,7 @@ def reinsert_eval(T, U, I0, h, p, unit_cost, fixed, consumption, *, table=None,
     a.policy_out = _dev_ptr(pol, "policy")
     a.value0_out = _dev_ptr(v0, "value0")
     a.mean_out = _dev_ptr(m, "mean")
-    ws = _workspace(lib.sdp_reinsert_workspace_bytes(ctypes.byref(a)), dev)
+    ws = _workspace(lib.sdp_reinsert_call_bytes(ctypes.byref(a)), dev)
     a.workspace, a.workspace_bytes = ws.data_ptr(), ws.numel()
     _check(lib.sdp_reinsert_eval(ctypes.byref(a), _stream(stream)))
     return {"value": val, "policy": pol, "value0": v0, "mean": m}

@@ -1052,23 +1052,28 @@ int sdp_split_grad_from_routes(int32_t n, int64_t S, const int32_t* tour, const 
 namespace {
 // the lane kernel keeps its decision bits in the workspace when the policy
 // is wanted
-bool reinsert_uses_lane(const sdp_reinsert_args* a) {
-  if (a->algo == SDP_REINSERT_AUTO && !a->value0_out &&
-      reinsert_chain_supported(a->T, a->U, a->end_cost_table != nullptr, a->n_routes, a->h, a->p, a->unit_cost))
-    return false;
-  return (a->algo == SDP_REINSERT_LANE || a->algo == SDP_REINSERT_AUTO) &&
-         !(a->n_routes > 0 && a->end_cost_table) &&
-         reinsert_lane_supported(a->T, a->U, a->n_routes);
+bool reinsert_uses_chain(const sdp_reinsert_args* a) {
+  return a->algo == SDP_REINSERT_AUTO && !a->value0_out &&
+         reinsert_chain_supported(a->T, a->U, a->end_cost_table != nullptr, a->n_routes, a->h, a->p, a->unit_cost);
 }
 size_t reinsert_scratch_bytes(const sdp_reinsert_args* a) {
-  return (reinsert_uses_lane(a) && a->policy_out && a->S > 0)
-             ? reinsert_lane_scratch_bytes(a->T, a->U) : 0;
+  const bool lane = (a->algo == SDP_REINSERT_LANE || a->algo == SDP_REINSERT_AUTO) &&
+                    !(a->n_routes > 0 && a->end_cost_table) &&
+                    reinsert_lane_supported(a->T, a->U, a->n_routes);
+  return (lane && a->policy_out && a->S > 0) ? reinsert_lane_scratch_bytes(a->T, a->U) : 0;
 }
+size_t reinsert_mean_bytes() { return align_up((size_t)kMeanBlocks * sizeof(double), 256); }
 }  // namespace
 
+// enough with and without value0_out: a caller may size once and set it later
 size_t sdp_reinsert_workspace_bytes(const sdp_reinsert_args* a) {
   if (!a || a->S < 0 || a->T < 1 || a->U < 0) return 0;
-  return align_up((size_t)kMeanBlocks * sizeof(double), 256) + reinsert_scratch_bytes(a);
+  return reinsert_mean_bytes() + reinsert_scratch_bytes(a);
+}
+
+size_t sdp_reinsert_call_bytes(const sdp_reinsert_args* a) {
+  if (!a || a->S < 0 || a->T < 1 || a->U < 0) return 0;
+  return reinsert_mean_bytes() + (reinsert_uses_chain(a) ? 0 : reinsert_scratch_bytes(a));
 }
 
 int sdp_reinsert_eval(const sdp_reinsert_args* a, void* stream) {
@@ -1109,8 +1114,8 @@ int sdp_reinsert_eval(const sdp_reinsert_args* a, void* stream) {
       return fail(SDP_ERR_INVALID_ARG, "value0_out must be a device pointer");
   }
   if (a->mean_out && !is_device_ptr(a->mean_out)) return fail(SDP_ERR_INVALID_ARG, "mean_out must be a device pointer");
-  const size_t need = sdp_reinsert_workspace_bytes(a);
-  const size_t scratch = reinsert_scratch_bytes(a);
+  const size_t need = sdp_reinsert_call_bytes(a);
+  const size_t scratch = need - reinsert_mean_bytes();
   int rc = (a->mean_out || scratch) ? check_ws(a->workspace, a->workspace_bytes, need) : SDP_OK;
   if (rc) return rc;
   uint32_t* status;
@@ -1125,8 +1130,7 @@ int sdp_reinsert_eval(const sdp_reinsert_args* a, void* stream) {
   r.S = a->S; r.fixed = a->fixed; r.table = a->end_cost_table; r.cons = a->consumption;
   r.value = a->value_out; r.policy = a->policy_out; r.value0 = a->value0_out; r.status = status;
   r.dscratch = scratch ? reinterpret_cast<uint32_t*>(
-                             static_cast<unsigned char*>(a->workspace) +
-                             align_up((size_t)kMeanBlocks * sizeof(double), 256))
+                             static_cast<unsigned char*>(a->workspace) + reinsert_mean_bytes())
                        : nullptr;
   r.mean_counter = a->mean_out ? mean_counter(static_cast<double*>(a->workspace)) : nullptr;
   prof_begin(st);
