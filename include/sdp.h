@@ -317,10 +317,14 @@ int sdp_split_backward(const sdp_split_args* fwd, const void* pred,
  * (hard capacity, device demands, demand rows of up to 512 staged bytes):
  * sdp_split_routes_workspace_bytes(a) is its workspace, 0 where it does not
  * run (SDP_ERR_UNSUPPORTED).  cost_out may be NULL (size the workspace with
- * the same cost_out as the call).
+ * the same cost_out as the call).  sdp_split_step_workspace_bytes(a) is the
+ * same where this pass takes about the time of the evaluation alone (n <= 50,
+ * or n <= 336 and all scenarios in one round of the kernel), else 0: what a
+ * training step uses that cannot know whether its backward will be called.
  * sdp_split_grad_from_routes turns them into d mean / d dist [(n+1)^2] times
  * *grad_mean (a device float, or a double that is rounded to float first). */
 size_t sdp_split_routes_workspace_bytes(const sdp_split_args* a);
+size_t sdp_split_step_workspace_bytes(const sdp_split_args* a);
 int sdp_split_eval_routes(const sdp_split_args* a, uint64_t* routes_out, void* stream);
 int sdp_split_grad_from_routes(int32_t n, int64_t S, const int32_t* tour, const uint64_t* routes,
                                const void* grad_mean, int32_t grad_is_double, float* grad_dist,

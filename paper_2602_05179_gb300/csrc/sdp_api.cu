@@ -995,6 +995,27 @@ size_t sdp_split_routes_workspace_bytes(const sdp_split_args* a) {
   return carve_split(a, nullptr, true, false).bytes + (a->cost_out ? 0 : sizeof(float) * (size_t)a->S);
 }
 
+// The adjoint's kernel counts routes behind the recursion and runs 16 to 24
+// warps per SM, PIPE 23 without counting, so a forward whose backward never
+// comes pays for the counts.  Its time over the separate forward's (memset,
+// preparation, PIPE, recomputation, two kernels for the mean) was, with 3 to 24
+// customers a route:
+//   tiles in one round of the kernel: n = 32..200 0.61-1.06, n = 250..336
+//     0.90-1.13 (1.05 with 6 customers a route or more but for n = 250 at 21
+//     tiles per SM, 1.11), n = 500 1.03-1.13;
+//   more rounds: n = 32 0.51-0.75, n = 50 0.78-1.01, n = 64 0.81-1.11,
+//     n = 100 0.91-1.55, n = 300 1.36-2.03 (S = 2 10^5: 231 -> 334 us).
+// One pass serves both where it costs the forward (next to) nothing.
+static bool routes_pay(const sdp_split_args* a) {
+  if (a->n <= 50) return true;
+  const int64_t tiles = (a->S + 31) / 32;
+  return a->n <= 336 && tiles <= (int64_t)adjoint_tmem_warps(a, false) * num_sms();
+}
+
+size_t sdp_split_step_workspace_bytes(const sdp_split_args* a) {
+  return a && a->n > 0 && a->S > 0 && routes_pay(a) ? sdp_split_routes_workspace_bytes(a) : 0;
+}
+
 int sdp_split_eval_routes(const sdp_split_args* args, uint64_t* routes_out, void* stream) {
   Demands dem;
   int rc = check_split(args, false, &dem);
