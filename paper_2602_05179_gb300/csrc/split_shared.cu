@@ -12,7 +12,8 @@
 // tour) pairs, tile by tile, are cut into one run per CTA, so that a CTA
 // stages two or three tiles of a launch of 313 tiles x 1,025 tours and
 // meets a barrier only between them; within a tile its warps claim tours
-// from a shared counter.
+// from a shared counter.  Launches of less than two tours per warp give each
+// tile its own CTAs instead (launch_split_shared).
 //
 // The recursion is that of split_pipe.cu (Eq. eqdpA in the K-form of
 // sdp_internal.cuh with a monotone deque per lane, entries (psi bits,
@@ -311,7 +312,7 @@ __device__ __forceinline__ void run_tour(int n, int Q, uint32_t tile, uint32_t r
 }
 
 template <typename QT>
-__global__ void __launch_bounds__(kSWarps * 32, 1) split_shared_kernel(PipeArgs a, int snap_step, int snap_count) {
+__global__ void __launch_bounds__(kSWarps * 32, 1) split_shared_kernel(PipeArgs a, int per_tile, int snap_step, int snap_count) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ uint32_t tile_inf;
   __shared__ int next_tour;
@@ -330,7 +331,12 @@ __global__ void __launch_bounds__(kSWarps * 32, 1) split_shared_kernel(PipeArgs 
   const int64_t tpt = (S + 31) / 32;
   // this CTA's run of the pairs (tile, tour), tile by tile
   const int64_t pairs = tpt * a.B;
-  const int64_t lo = pairs * blockIdx.x / gridDim.x, hi = pairs * (blockIdx.x + 1) / gridDim.x;
+  int64_t lo = pairs * blockIdx.x / gridDim.x, hi = pairs * (blockIdx.x + 1) / gridDim.x;
+  if (per_tile > 0) {  // or its share of one tile's tours
+    const int64_t t = blockIdx.x / per_tile, j = blockIdx.x % per_tile;
+    lo = t * a.B + a.B * j / per_tile;
+    hi = t * a.B + a.B * (j + 1) / per_tile;
+  }
   const Snapshots snap{(tile + (uint32_t)(n * 32 * (int)sizeof(QT)) + 15u) & ~15u, snap_step, snap_count, &snap_ready};
   uint32_t any_inf = 0, any_fb = 0;
   bool neg = false;
@@ -431,7 +437,7 @@ size_t shared_smem(int n, int Q) {
 }
 
 template <typename QT>
-int launch_s(const PipeArgs& a, int grid, cudaStream_t st) {
+int launch_s(const PipeArgs& a, int grid, int per_tile, cudaStream_t st) {
   auto k = split_shared_kernel<QT>;
   // tour 0's states: as many as fit, every 8 positions at best (the last one
   // before position n)
@@ -445,7 +451,7 @@ int launch_s(const PipeArgs& a, int grid, cudaStream_t st) {
   const size_t smem = tiles + (size_t)count * kSStateBytes;
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
-  k<<<grid, kSWarps * 32, smem, st>>>(a, step, count);
+  k<<<grid, kSWarps * 32, smem, st>>>(a, per_tile, step, count);
   return (int)cudaGetLastError();
 }
 
@@ -457,10 +463,30 @@ bool shared_supported(int n, int Q, int B) {
          shared_smem(n, Q) <= kSSmemMax;
 }
 
+// Below two tours per warp of the chip, a run of pairs that crosses from one
+// tile into the next takes a barrier and one more tour's time for a few pairs,
+// and a run of at least 32 leaves SMs without any where there are few: there
+// every tile gets an equal number of CTAs, as many as there are SMs for, if its
+// warps then take fewer tours one after the other than the worst run would, or
+// as many on no fewer SMs.  Against runs, where these took one tour more than
+// the pipelined kernel had (n = 1000, Q = 100): 100 tours x 16 tiles 423 -> 220
+// us (pipelined 300), 64 x 1 257 -> 182 (222), 100 x 63 562 -> 443 (613).
 int launch_split_shared(const PipeArgs& a, cudaStream_t st) {
-  const int64_t pairs = (a.S + 31) / 32 * a.B;
-  const int grid = (int)imin64(num_sms(), (pairs + kSWarps - 1) / kSWarps);
-  return a.Q <= 254 ? launch_s<uint8_t>(a, grid, st) : launch_s<uint16_t>(a, grid, st);
+  const int64_t tiles = (a.S + 31) / 32, pairs = tiles * a.B, sms = num_sms();
+  int per_tile = 0;
+  int64_t grid = imin64(sms, (pairs + kSWarps - 1) / kSWarps);
+  if (pairs < 2 * kSWarps * sms) {  // so tiles < SMs, as B >= 64, and a run crosses once
+    const int64_t run = (pairs + grid - 1) / grid;
+    const int64_t run_tours = tiles == 1 ? (run + kSWarps - 1) / kSWarps : (run - 2) / kSWarps + 2;
+    const int64_t share = imin64(a.B, sms / tiles);
+    const int64_t own_tours = ((a.B + share - 1) / share + kSWarps - 1) / kSWarps;
+    if (own_tours < run_tours || (own_tours == run_tours && tiles * share >= grid)) {
+      per_tile = (int)share;
+      grid = tiles * share;
+    }
+  }
+  return a.Q <= 254 ? launch_s<uint8_t>(a, (int)grid, per_tile, st)
+                    : launch_s<uint16_t>(a, (int)grid, per_tile, st);
 }
 
 }  // namespace sdp

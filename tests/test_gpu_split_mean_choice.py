@@ -10,10 +10,10 @@ pytestmark = pytest.mark.gpu
 
 
 def _round(n, Q):
-    """Scenarios of one round: 24 warps per SM where 24 row shares fit the
-    tensor memory, else 16."""
-    words = n if Q <= 254 else 2 * n
-    warps = 24 if words <= 4 * ((512 // 6) & ~3) else 16
+    """Scenarios of one round: as many warps per SM, 16 to 24, as have tensor
+    memory columns for a row (rows take a multiple of four)."""
+    words = ((n if Q <= 254 else 2 * n) + 15) // 16 * 4
+    warps = max(w for w in range(16, 25) if words <= (512 // ((w + 3) // 4) & ~3))
     return 32 * warps * torch.cuda.get_device_properties(0).multi_processor_count
 
 
@@ -23,7 +23,7 @@ def _round(n, Q):
     (51, 100, 1, False),
     (100, 300, 0, True),
     (100, 300, 1, False),
-    (200, 300, 0, True),      # rows of 400 bytes: 16 warps
+    (200, 300, 0, True),      # rows of 400 bytes: 20 warps
     (200, 300, 1, False),
     (336, 100, 0, True),
     (336, 100, 1, False),
