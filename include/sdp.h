@@ -256,7 +256,10 @@ int sdp_split_eval_noalloc(const sdp_split_args* a, void* stream);
  * ties to the smallest p at every (k, i), then to the fewest routes.
  *   a:           as for sdp_split_eval, with pred_out = NULL, hard capacity,
  *                device demands, algo SDP_ALGO_AUTO (one warp per scenario,
- *                the route counts across its lanes) or SDP_ALGO_PLAIN (one
+ *                over the positions that at most max_routes routes allow, or
+ *                all positions with the route counts across its lanes where
+ *                the fleet has much slack or the tour is long) or
+ *                SDP_ALGO_PLAIN (one
  *                thread per scenario, every feasible p of every layer; the
  *                same FP32 operations and bits); cost_out [S] fp32 (+inf
  *                where no split into at most max_routes routes fits Q, or a

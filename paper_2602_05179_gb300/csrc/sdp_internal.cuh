@@ -350,6 +350,8 @@ struct SplitFleetArgs {
   uint16_t* dscratch;        // warp kernels with routes: fleet_dscratch_elems
   uint32_t* fb_list;         // warp kernel: flagged scenarios; plain: NULL = all S
   uint32_t* fb_count;
+  uint32_t* loose;           // set by the band kernel: the deque kernel takes the call's scenarios
+  uint32_t loose_load;       // ... where a sample's demands add up to less than this (0: never)
   float* kscratch;           // plain: [nslots * 2 * (n+1)]
   uint16_t* pscratch;        // plain with routes: [nslots * K * n]
   int64_t nslots;
@@ -359,8 +361,12 @@ struct FleetConfig {
   int warps;  // warps per CTA (0: the tour's records do not fit)
   int grid;
   bool band;  // the band kernel, which also recomputes what it flags
+  // band: the sample's load below which the deque kernel takes the scenarios
+  // (0: never), and that kernel's shape
+  uint32_t loose_load;
+  int loose_warps, loose_grid;
 };
-FleetConfig fleet_config(int n, int K, int64_t S);
+FleetConfig fleet_config(int n, int Q, int K, int64_t S);
 size_t fleet_dscratch_elems(int n, int K, const FleetConfig& c);
 int launch_split_fleet(const SplitFleetArgs& a, const FleetConfig& c, cudaStream_t st);
 int launch_split_fleet_plain(const SplitFleetArgs& a, cudaStream_t st);

@@ -31,9 +31,12 @@
 //   n = 500, K = 42, S = 65,536: 1.12 ms where the deque kernel
 // below, which steps every layer through every position, took 5.43 ms and
 // 0.32 ms of recomputation.
+//   A fleet with much slack makes the band the whole tour: such calls it leaves
+// to the deque kernel (fleet_loose_load), which hands back the scenarios whose
+// deque outgrows its ring.
 //
-// split_fleet_kernel (longer tours): one warp per scenario, the layers across
-// its lanes:
+// split_fleet_kernel (longer tours, calls with much slack): one warp per
+// scenario, the layers across its lanes:
 // lane l's slot j holds layer k = 32 j + l + 1 (two slots: K <= 64).  Every
 // lane walks the same positions i = 1..n in lockstep, so the demand of s_i
 // and the tour record are broadcast loads; layer k's input psi_{k-1}(i-1) =
@@ -55,6 +58,7 @@
 
 #include <algorithm>
 
+#include "dependent.cuh"
 #include "sdp_internal.cuh"
 
 namespace sdp {
@@ -147,6 +151,9 @@ __global__ void __launch_bounds__(kFMaxWarps * 32) split_fleet_kernel(SplitFleet
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int n = a.n, Q = a.Q, K = a.K;
+  dep_launch();
+  const bool shared_call = a.loose_load != 0u;  // with the band kernel, which chose
+  if (shared_call && *a.loose == 0u) return;
   // shared: (a_i, ce_i) and columns of the tour | per warp: KS rings,
   // route boundaries
   float2* rec = reinterpret_cast<float2*>(smem);
@@ -169,6 +176,16 @@ __global__ void __launch_bounds__(kFMaxWarps * 32) split_fleet_kernel(SplitFleet
   uint16_t* dsc = ROUTES ? a.dscratch + wslot * (int64_t)n * 32 * KS : nullptr;
   bool neg = false, any_fb = false, any_inf = false;
   for (int64_t s = wslot; s < a.S; s += (int64_t)gridDim.x * nw) {
+    if (shared_call && s != wslot) {
+      // rings outgrow on a tour more than on a scenario: where one in eight so
+      // far has, the rest goes to the band kernel too
+      uint32_t back = 0u;
+      if (lane == 0) back = __ldcg(a.fb_count);
+      if ((int64_t)__shfl_sync(0xffffffffu, back, 0) > 16 + s / 8) {
+        if (lane == 0) a.fb_list[atomicAdd(a.fb_count, 1u)] = (uint32_t)s;
+        continue;
+      }
+    }
     const int32_t* qrow = a.demands + s * n;
     FleetDeque dq[KS];
 #pragma unroll
@@ -212,6 +229,7 @@ __global__ void __launch_bounds__(kFMaxWarps * 32) split_fleet_kernel(SplitFleet
         }
         Lc = Lnew;
       }
+      if (shared_call && __any_sync(0xffffffffu, dq[0].full || dq[KS - 1].full)) break;
     }
     // the best layer k <= K, fewest routes on ties
     float best = CUDART_INF_F;
@@ -484,6 +502,7 @@ constexpr int kBandMaxWarps = 24;
 constexpr int kBandMinWarps = 8;   // per SM: fewer hide too little latency
 constexpr int kBandWindow = 32;    // longest window of the narrow form
 constexpr int kBandNarrow = 4, kBandWide = 16;  // positions per block minimum
+constexpr int kBandSample = 8;     // scenarios that the choice of kernel looks at
 
 // CTA: a_{p+1} and ce_i [n+1] floats each, columns [n]; per warp: prefix
 // loads, psi and block minima [n+1 .. +16] (each on 16 bytes), window starts [n+1] uint16, and
@@ -497,7 +516,8 @@ __host__ __device__ constexpr size_t band_per_warp(int n, int K) {
 }
 
 // B: positions per block minimum.  LIST: the flagged scenarios (fb_list);
-// otherwise all, flagging those with a window above kBandWindow.
+// otherwise all, flagging those with a window above kBandWindow, or none where
+// a sample of the scenarios says that the fleet has much slack (loose_load).
 template <int B, bool LIST, bool ROUTES>
 __global__ void __launch_bounds__(kBandMaxWarps * 32) split_fleet_band_kernel(SplitFleetArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -515,6 +535,25 @@ __global__ void __launch_bounds__(kBandMaxWarps * 32) split_fleet_band_kernel(Sp
   uint16_t* lo_of = pm + n + 1;      // [m]: the first position that m more routes take to n
   uint16_t* hi_of = lo_of + K + 2;   // [k]: the last position that k routes reach
   uint16_t* bound = hi_of + K + 2;   // route k covers positions bound[k] + 1 .. bound[k+1]
+  if (LIST) dep_wait();
+  if (!LIST && a.loose_load) {
+    __shared__ uint32_t load;
+    if (threadIdx.x == 0) load = 0u;
+    __syncthreads();
+    for (int j = warp; j < kBandSample; j += nw) {
+      const int32_t* q = a.demands + (a.S - 1) * j / (kBandSample - 1) * n;
+      uint32_t v = 0u;
+#pragma unroll 8
+      for (int k = lane; k < n; k += 32) v += (uint32_t)min(max(__ldg(q + k), 0), Q + 1);
+      v = __reduce_add_sync(kAll, v);
+      if (lane == 0) atomicAdd(&load, v);
+    }
+    __syncthreads();
+    if (load < a.loose_load) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) *a.loose = 1u;
+      return;
+    }
+  }
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     const StepRec r = a.rec[k];
     as[k] = r.a;
@@ -747,6 +786,12 @@ int launch_fleet_k(const SplitFleetArgs& a, int warps, int grid, cudaStream_t st
   return (int)cudaGetLastError();
 }
 
+int launch_deque(const SplitFleetArgs& a, int warps, int grid, cudaStream_t st) {
+  if (a.K <= 32)
+    return a.route ? launch_fleet_k<1, true>(a, warps, grid, st) : launch_fleet_k<1, false>(a, warps, grid, st);
+  return a.route ? launch_fleet_k<2, true>(a, warps, grid, st) : launch_fleet_k<2, false>(a, warps, grid, st);
+}
+
 template <bool ROUTES>
 int launch_band(const SplitFleetArgs& a, const FleetConfig& c, cudaStream_t st) {
   const size_t smem = band_head(a.n) + band_per_warp(a.n, a.K) * c.warps;
@@ -757,54 +802,87 @@ int launch_band(const SplitFleetArgs& a, const FleetConfig& c, cudaStream_t st) 
     e = cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
   narrow<<<c.grid, c.warps * 32, smem, st>>>(a);
-  wide<<<c.grid, c.warps * 32, smem, st>>>(a);
-  return (int)cudaGetLastError();
+  if (a.loose_load) {
+    const int d = launch_deque(a, c.loose_warps, c.loose_grid, st);
+    if (d) return d;
+  }
+  // placed while the deque kernel finds that it has nothing to do; placed early
+  // behind the narrow form it slows that one (n = 500, K = 42: 1128 -> 1153 us)
+  return (int)launch_dependent(a.loose_load != 0u, wide, c.grid, c.warps * 32, smem, st, a);
+}
+
+// The deque kernel's shape: one CTA per SM with as many warps as its shared
+// memory holds; fewer CTAs when there are fewer scenarios.
+void deque_shape(int n, int K, int64_t S, int* warps, int* grid) {
+  const size_t budget = 226 * 1024;  // dynamic shared memory of one CTA per SM
+  const size_t head = fleet_head(n);
+  const int w = head >= budget ? 0 : (int)((budget - head) / fleet_per_warp(K <= 32 ? 1 : 2));
+  *warps = w > kFMaxWarps ? kFMaxWarps : w;
+  if (*warps < 1) return;
+  const int64_t need = (S + *warps - 1) / *warps;
+  *grid = (int)imin64(need < 1 ? 1 : need, (int64_t)num_sms());
+}
+
+// The load of the kBandSample scenarios below which the deque kernel takes a
+// call rather than the band kernel, as a multiple of Q: routes that they need
+// at least, kBandSample times their mean m.
+//   The band of a scenario holds about n (K - m) states.  On 65,536 scenarios
+// (n = 31..500, K up to 64, windows of 4 to n positions, random and sweep tours)
+// the band kernel takes about 12.3 K + 0.25 n (K - m) us beyond what both do,
+// 0.34 n (K - m) for windows of n / 3 positions and more; the deque kernel 6.5 n
+// (K <= 32) or 10.3 n (two layers a lane) while its rings hold, which the lines
+// below take 5% higher.  Everything in the band, K = 64 and windows of 32 of
+// n = 100 took 3.45 ms, the deque kernel 1.30; n = 300, window 46: 5.71 and
+// 3.70.  A tight fleet (n = 500, K = 42, 39 to 42 needed): 1.12 and 5.75.  With
+// the choice, of 1,500 sizes from S = 200 on none took more than 1.07 times the
+// deque kernel's time (one 1.13); tight fleets pay 3 us for it.  Where rings
+// outgrow (windows of 24 to n / 3 positions on long tours) the deque kernel's
+// share until the scenarios are handed back is up to 12% of the band's time.
+uint32_t fleet_loose_load(int n, int Q, int K) {
+  const double deque = (K <= 32 ? 27.0 : 43.0) - 49.0 * K / n;  // per position, in units of 0.25 us
+  const double m = std::max(K - deque, std::min(3.0, K - deque / 1.35));
+  // (less than one route: hardly a call, and the choice costs each call a launch)
+  return m >= 1.0 ? (uint32_t)(kBandSample * std::min(m, (double)K + 1.0) * Q) : 0u;
 }
 
 }  // namespace
 
-// One CTA per SM with as many warps as its shared memory holds (up to 16);
-// fewer CTAs when there are fewer scenarios.
-FleetConfig fleet_config(int n, int K, int64_t S) {
+// The band kernel: one CTA per SM with as many warps as its shared memory
+// holds, spread over all SMs when there are few scenarios; else the deque
+// kernel alone.
+FleetConfig fleet_config(int n, int Q, int K, int64_t S) {
+  FleetConfig c{};
   if (band_head(n) + band_per_warp(n, K) * kBandMinWarps <= 226 * 1024) {
     int warps = (int)((226 * 1024 - band_head(n)) / band_per_warp(n, K));
     warps = warps > kBandMaxWarps ? kBandMaxWarps : warps;
     // few scenarios: as many SMs as possible
     const int64_t share = (S + num_sms() - 1) / num_sms();
-    FleetConfig c{};
     c.band = true;
     c.warps = (int)imin64(warps, share < 1 ? 1 : share);
     const int64_t need = (S + c.warps - 1) / c.warps;
     c.grid = (int)imin64(need < 1 ? 1 : need, (int64_t)num_sms());
+    c.loose_load = fleet_loose_load(n, Q, K);
+    if (c.loose_load) deque_shape(n, K, S, &c.loose_warps, &c.loose_grid);
+    if (c.loose_warps < 1) c.loose_load = 0u;
     return c;
   }
-  const int ks = K <= 32 ? 1 : 2;
-  const size_t budget = 226 * 1024;  // dynamic shared memory of one CTA per SM
-  const size_t head = fleet_head(n);
-  int warps = head >= budget ? 0 : (int)((budget - head) / fleet_per_warp(ks));
-  warps = warps > kFMaxWarps ? kFMaxWarps : warps;
-  FleetConfig c{};
-  c.warps = warps;
-  if (warps < 1) return c;
-  const int64_t need = (S + warps - 1) / warps;
-  c.grid = (int)imin64(need < 1 ? 1 : need, (int64_t)num_sms());
+  deque_shape(n, K, S, &c.warps, &c.grid);
   return c;
 }
 
+// the band's rows (floats) and the deque kernel's route deltas share it, one
+// kernel after the other
 size_t fleet_dscratch_elems(int n, int K, const FleetConfig& c) {
-  if (c.band) return (size_t)c.grid * c.warps * (size_t)K * (size_t)(n + 1) * 2;  // floats
-  const int ks = K <= 32 ? 1 : 2;
-  return (size_t)c.grid * c.warps * (size_t)n * 32 * ks;
+  const size_t deltas = (size_t)n * 32 * (K <= 32 ? 1 : 2);
+  if (!c.band) return (size_t)c.grid * c.warps * deltas;
+  const size_t rows = (size_t)c.grid * c.warps * (size_t)K * (size_t)(n + 1) * 2;
+  return c.loose_load ? std::max(rows, (size_t)c.loose_grid * c.loose_warps * deltas) : rows;
 }
 
 int launch_split_fleet(const SplitFleetArgs& a, const FleetConfig& c, cudaStream_t st) {
   if (c.warps < 1) return (int)cudaErrorInvalidValue;
   if (c.band) return a.route ? launch_band<true>(a, c, st) : launch_band<false>(a, c, st);
-  if (a.K <= 32)
-    return a.route ? launch_fleet_k<1, true>(a, c.warps, c.grid, st)
-                   : launch_fleet_k<1, false>(a, c.warps, c.grid, st);
-  return a.route ? launch_fleet_k<2, true>(a, c.warps, c.grid, st)
-                 : launch_fleet_k<2, false>(a, c.warps, c.grid, st);
+  return launch_deque(a, c.warps, c.grid, st);
 }
 
 bool fleet_rescue_supported(int n) { return fleet_rescue_head(n) + fleet_rescue_per_warp(n) <= 200u * 1024u; }
