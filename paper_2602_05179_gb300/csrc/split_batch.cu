@@ -210,13 +210,16 @@ void drop_graph(sdp_plan* p) {
   p->exec = nullptr;
 }
 
+// What the timings depend on: the sizes, and which kernels the shapes -2 and -1
+// stand for in this plan.  The number behind `kernels` is raised when a kernel takes another's
+// place behind a shape, so that entries timed before do not match.
 std::string cache_key(const sdp_plan* p) {
   cudaDeviceProp prop;
   cudaGetDeviceProperties(&prop, p->device);
-  char buf[256];
-  snprintf(buf, sizeof(buf), "%s|sm%d|B%d|S%lld|Q%d|nmax%d|sumn%lld", prop.name,
-           prop.multiProcessorCount, p->B, (long long)p->S, p->Q, p->n_max,
-           (long long)p->sum_n);
+  char buf[320];
+  snprintf(buf, sizeof(buf), "%s|sm%d|B%d|S%lld|Q%d|nmax%d|sumn%lld|kernels2|shared%d|pipe%d|stream%d",
+           prop.name, prop.multiProcessorCount, p->B, (long long)p->S, p->Q, p->n_max,
+           (long long)p->sum_n, p->shared ? 1 : 0, p->d_pq ? 1 : 0, p->d_qt ? 1 : 0);
   std::string k(buf);
   for (char& c : k)
     if (c == ' ') c = '_';
