@@ -310,6 +310,15 @@ size_t sdp_saa_search_desc_size(void) { return sizeof(sdp_saa_search_desc); }
 
 int sdp_saa_search_autotune(sdp_saa_search* s, void* stream, const char* cache_path) {
   if (!s) return sfail(SDP_ERR_INVALID_ARG, "search is NULL");
+  // timed on tours that the search scores: the last iteration's, or, before
+  // any, the first's (the plan's slots all hold tour 0 then, which a kernel
+  // that resumes from shared beginnings hardly runs)
+  if (s->iter == 0 && on_own_device(s)) {
+    saa_candidates_kernel<<<s->B + 1, 128, 0, static_cast<cudaStream_t>(stream)>>>(
+        s->d_cur, s->d_cand, s->n, s->B, s->seed, s->iter, s->moves);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return scuda(e, "search candidates");
+  }
   return plan_autotune(s->plan, stream, cache_path, 16);
 }
 
