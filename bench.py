@@ -524,8 +524,9 @@ def operators(api, wl, dev, only="", steps=0, checks=True):
 
 
 def op_reinsert(c, out):
-    """Reinsertion T=60, U=200, S=10^6 (ALU bound): the default kernel (one
-    scenario per lane) against the one-scenario-per-warp kernel."""
+    """Reinsertion T=60, U=200, S=10^6: the default kernel (the reachable
+    states, one scenario per lane) against the one-scenario-per-warp kernel,
+    which evaluates every state."""
     import torch
     rs = c.wl.REINSERT_C3
     cons = c.wl.reinsert_consumption_device(rs, c.dev)
@@ -539,12 +540,9 @@ def op_reinsert(c, out):
     r = run("auto")
     wms, wkms = _timed(lambda: run("warp"), 5)
     rw = run("warp")
-    rel = 2.0 * (rs.U + 1) * rs.T * rs.S
-    line = {"value": rel / (ms / 1e3), "unit": "relaxations/s",
-            "scenarios_per_s": rs.S / (ms / 1e3), "ms_per_step": ms, "kernel_ms": kms,
+    line = {"value": rs.S / (ms / 1e3), "unit": "scenarios/s", "ms_per_step": ms, "kernel_ms": kms,
             "kernel": "reinsert_chain_kernel (reachable states, one scenario per lane)",
-            # value counts the states of the whole recursion; the roofline credits
-            # the at most t + 1 of them that day t can start in
+            # credits the at most t + 1 states that day t can start in
             "roofline": c.alu_roof(2 * rs.S * sum(min(t + 1, rs.U + 1) for t in range(rs.T)), kms),
             "vs_plain": {"kernel": "reinsert_kernel (one scenario per warp)",
                          "ms_per_step": wms, "kernel_ms": wkms, "speedup": wkms / kms,
@@ -563,7 +561,7 @@ def op_reinsert(c, out):
 
 
 def op_routes(c, out):
-    """Reinsertion with K = 4 route options per day (ALU bound)."""
+    """Reinsertion with K = 4 route options per day."""
     import torch
     rr = c.wl.REINSERT_ROUTES
     cons = c.wl.reinsert_consumption_device(rr, c.dev)
@@ -580,9 +578,7 @@ def op_routes(c, out):
     wms, wkms = _timed(lambda: run("warp"), c.steps or 10)
     rw = run("warp")
     same = all(bool(torch.equal(r[k], rw[k])) for k in ("value", "policy"))
-    rel = float(rr.U + 1) * rr.T * (K + 1) * rr.S  # (state, action) pairs
-    line = {"value": rel / (ms / 1e3), "unit": "relaxations/s",
-            "scenarios_per_s": rr.S / (ms / 1e3), "ms_per_step": ms, "kernel_ms": kms,
+    line = {"value": rr.S / (ms / 1e3), "unit": "scenarios/s", "ms_per_step": ms, "kernel_ms": kms,
             "kernel": "reinsert_chain_kernel (route options, reachable states, one scenario per lane)",
             "roofline": c.alu_roof(2 * rr.S * (K + 1) * sum(min(t + 1, rr.U + 1) for t in range(rr.T)), kms),
             "vs_warp": {"kernel": "reinsert_routes_kernel (one scenario per warp)", "ms_per_step": wms,
@@ -704,12 +700,31 @@ def op_soft(c, out):
     out["split_soft_n500_S1e6_beta10"] = line
 
 
+def band_states(q, tour, Q, K):
+    """States (k, i) of each scenario from which a split into at most K routes
+    can still finish: i lies between what k routes reach from the start and
+    what K - k reach back from the end (0 where no such split exists)."""
+    n = len(tour)
+    out = np.zeros(len(q), np.int64)
+    for s, row in enumerate(np.asarray(q, np.int64)[:, np.asarray(tour) - 1]):
+        if (row > Q).any():
+            continue
+        L = np.concatenate([[0], np.cumsum(row)])
+        hi, lo = [0], [n]
+        for _ in range(K):
+            hi.append(int(np.searchsorted(L, L[hi[-1]] + Q, side="right")) - 1)
+            lo.append(int(np.searchsorted(L, L[lo[-1]] - Q, side="left")))
+        if lo[K] == 0:
+            out[s] = sum(max(0, hi[k] - max(lo[K - k], 1) + 1) for k in range(1, K + 1))
+    return out
+
+
 def op_fleet(c, out):
     """Fleet-limited Split (at most K = 42 routes) on the Split benchmark's
     recipe (n = 500, Q = 200, U{1..30}) with S = 65,536: the limit binds
-    (about 39-42 routes are needed).  Work unit: the K-layer relaxations,
-    K x feasible arcs per scenario (2 ops each); the plain comparison runs
-    every feasible p of every layer, one thread per scenario, on 4,096
+    (about 39-42 routes are needed).  The kernel evaluates the band of states
+    that K routes leave, counted here on 256 scenarios; the plain comparison
+    runs every feasible p of every layer, one thread per scenario, on 4,096
     scenarios."""
     import dataclasses
     import torch
@@ -719,9 +734,6 @@ def op_fleet(c, out):
     t = torch.from_numpy(tour).to(c.dev)
     cc = torch.from_numpy(xy).to(c.dev)
     q = c.wl.split_demands_device(spec, c.dev, 0, S)
-    arcs, total = c.api.split_count_arcs(t, spec.Q, q, coords=cc, per_scenario=False)
-    torch.cuda.synchronize()
-    rel = float(total) * K
     fn = lambda: c.api.split_fleet_eval(t, spec.Q, q, K, coords=cc)
     ms, kms = _timed(fn, c.steps or 5)
     c.api.status()
@@ -735,15 +747,16 @@ def op_fleet(c, out):
     torch.cuda.synchronize()
     same = all(bool(torch.equal(r[k][:Sp], rp[k])) for k in ("cost", "nroutes", "route"))
     fin = torch.isfinite(r["cost"])
+    states = band_states(q[:: S // 256].cpu().numpy(), tour, spec.Q, K).mean()
     line = {"value": S / (ms / 1e3), "unit": "scenarios/s", "ms_per_step": ms, "kernel_ms": kms,
             "kernel": "split_fleet_band_kernel (one warp per scenario, positions across lanes)",
             "max_routes": K, "feasible_frac": float(fin.float().mean()),
             "flagged_recomputed": fell_back,
             "recompute": "scenarios with windows of more than 32 positions: the same kernel in wider "
                          "blocks, inside ms_per_step",
-            # of the whole recursion; the kernel evaluates the band that K routes leave
-            "layer_relaxations_per_s": rel / (kms / 1e3),
-            "roofline": c.alu_roof(2 * rel, kms),
+            # demands in; cost, route count and each customer's route out
+            "roofline": c.hbm_roof(S * (spec.n * 4 + 4 + 4 + spec.n), kms),
+            "band_states_per_scenario": float(states), "states_per_s": float(states) * S / (kms / 1e3),
             "vs_plain": {"path": "one thread per scenario, every feasible p of every layer",
                          "sample": Sp, "kernel_ms": pkms,
                          "speedup_per_scenario": (pkms / Sp) / (kms / S),
@@ -878,11 +891,14 @@ def op_saa(c, out):
             "ms_per_iteration": ms / iters, "iterations": iters,
             "scenario_evaluations_per_s": evals * spec.S / (ms / 1e3),
             "arcs_per_s": arcs / (ms / 1e3), "arcs": arcs,
-            "roofline": c.alu_roof(2 * arcs, ms / iters * iters),
+            # the scenarios in, the costs out and in again for the means
+            "roofline": c.hbm_roof(iters * (spec.S * spec.n * 4 + (c.wl.SAA_B + 1) * spec.S * 8), ms),
             "best_mean_first": float(tr[0]), "best_mean_last": float(tr[-1]),
             "improving_iterations": int((acc >= 0).sum()),
             "launch": shape}
-    line["roofline"]["note"] = "whole iterations (moves, plan replay, selection) timed"
+    line["roofline"]["note"] = ("whole iterations (moves, plan replay, selection) timed; bound by instruction "
+                                "issue, and arcs of beginnings that a neighbour shares with the current "
+                                "tour are scored without being run")
     if c.checks:
         import oracle
         ft = final_tour.cpu().numpy()
