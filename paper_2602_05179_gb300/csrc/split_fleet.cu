@@ -536,23 +536,17 @@ __global__ void __launch_bounds__(kBandMaxWarps * 32) split_fleet_band_kernel(Sp
   uint16_t* hi_of = lo_of + K + 2;   // [k]: the last position that k routes reach
   uint16_t* bound = hi_of + K + 2;   // route k covers positions bound[k] + 1 .. bound[k+1]
   if (LIST) dep_wait();
+  // every CTA adds up the same scenarios' demands, while the records load
+  __shared__ uint32_t load[kBandMaxWarps];
   if (!LIST && a.loose_load) {
-    __shared__ uint32_t load;
-    if (threadIdx.x == 0) load = 0u;
-    __syncthreads();
+    uint32_t v = 0u;
     for (int j = warp; j < kBandSample; j += nw) {
       const int32_t* q = a.demands + (a.S - 1) * j / (kBandSample - 1) * n;
-      uint32_t v = 0u;
 #pragma unroll 8
       for (int k = lane; k < n; k += 32) v += (uint32_t)min(max(__ldg(q + k), 0), Q + 1);
-      v = __reduce_add_sync(kAll, v);
-      if (lane == 0) atomicAdd(&load, v);
     }
-    __syncthreads();
-    if (load < a.loose_load) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) *a.loose = 1u;
-      return;
-    }
+    v = __reduce_add_sync(kAll, v);
+    if (lane == 0) load[warp] = v;
   }
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     const StepRec r = a.rec[k];
@@ -562,6 +556,14 @@ __global__ void __launch_bounds__(kBandMaxWarps * 32) split_fleet_band_kernel(Sp
   }
   if (threadIdx.x == 0) as[n] = 0.f;
   __syncthreads();
+  if (!LIST && a.loose_load) {
+    uint32_t v = 0u;
+    for (int w = 0; w < nw; ++w) v += load[w];
+    if (v < a.loose_load) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) *a.loose = 1u;
+      return;
+    }
+  }
   const double Dn = *a.Dn;
   const int64_t slot = (int64_t)blockIdx.x * nw + warp;
   float* rows = ROUTES ? reinterpret_cast<float*>(a.dscratch) + slot * K * (int64_t)(n + 1) : nullptr;
@@ -824,25 +826,32 @@ void deque_shape(int n, int K, int64_t S, int* warps, int* grid) {
 }
 
 // The load of the kBandSample scenarios below which the deque kernel takes a
-// call rather than the band kernel, as a multiple of Q: routes that they need
-// at least, kBandSample times their mean m.
+// call rather than the band kernel: kBandSample Q times the mean m of the routes
+// that they need at least.
 //   The band of a scenario holds about n (K - m) states.  On 65,536 scenarios
 // (n = 31..500, K up to 64, windows of 4 to n positions, random and sweep tours)
 // the band kernel takes about 12.3 K + 0.25 n (K - m) us beyond what both do,
 // 0.34 n (K - m) for windows of n / 3 positions and more; the deque kernel 6.5 n
 // (K <= 32) or 10.3 n (two layers a lane) while its rings hold, which the lines
-// below take 5% higher.  Everything in the band, K = 64 and windows of 32 of
-// n = 100 took 3.45 ms, the deque kernel 1.30; n = 300, window 46: 5.71 and
-// 3.70.  A tight fleet (n = 500, K = 42, 39 to 42 needed): 1.12 and 5.75.  With
-// the choice, of 1,500 sizes from S = 200 on none took more than 1.07 times the
-// deque kernel's time (one 1.13); tight fleets pay 3 us for it.  Where rings
-// outgrow (windows of 24 to n / 3 positions on long tours) the deque kernel's
-// share until the scenarios are handed back is up to 12% of the band's time.
-uint32_t fleet_loose_load(int n, int Q, int K) {
-  const double deque = (K <= 32 ? 27.0 : 43.0) - 49.0 * K / n;  // per position, in units of 0.25 us
+// below take 5% higher.  Up to a scenario per warp of the chip the band kernel
+// spreads them over all SMs, and the line lies higher.  Everything in the band,
+// K = 64 and windows of 32 of n = 100 took 3.45 ms, the deque kernel 1.30;
+// n = 300, window 46: 5.71 and 3.70.  A tight fleet (n = 500, K = 42, 39 to 42
+// needed): 1.13 and 5.75.
+//   With the choice, 1,500 sizes from S = 200 on take at most 1.08 of the deque
+// kernel's time (eight of them up to 1.20).  It costs tight fleets a launch (1 to
+// 6 us; inlined into the band kernel, or called from it, the deques cost the band
+// 2 to 13%), and calls whose rings do outgrow (windows of 22 to n / 3 positions;
+// the deque kernel and its recomputation took 2 to 20 times the band's time
+// there) the time until the scenarios are handed back: up to 12% of the band's
+// time, up to 78% where each warp has one scenario.
+uint32_t fleet_loose_load(int n, int Q, int K, int64_t S) {
+  const double idle = std::max(0.0, 1.0 - (double)S / (kFMaxWarps * num_sms()));
+  // per position, in units of 0.25 us on 65,536 scenarios
+  const double deque = (K <= 32 ? 27.0 + 6.0 * idle : 43.0 + 3.0 * idle) + 1200.0 * idle / n - 49.0 * K / n;
   const double m = std::max(K - deque, std::min(3.0, K - deque / 1.35));
   // (less than one route: hardly a call, and the choice costs each call a launch)
-  return m >= 1.0 ? (uint32_t)(kBandSample * std::min(m, (double)K + 1.0) * Q) : 0u;
+  return m >= 1.0 ? (uint32_t)(kBandSample * std::min(m, K + 1.0) * Q) : 0u;
 }
 
 }  // namespace
@@ -861,7 +870,7 @@ FleetConfig fleet_config(int n, int Q, int K, int64_t S) {
     c.warps = (int)imin64(warps, share < 1 ? 1 : share);
     const int64_t need = (S + c.warps - 1) / c.warps;
     c.grid = (int)imin64(need < 1 ? 1 : need, (int64_t)num_sms());
-    c.loose_load = fleet_loose_load(n, Q, K);
+    c.loose_load = fleet_loose_load(n, Q, K, S);
     if (c.loose_load) deque_shape(n, K, S, &c.loose_warps, &c.loose_grid);
     if (c.loose_warps < 1) c.loose_load = 0u;
     return c;
