@@ -500,9 +500,11 @@ void sdp_saa_search_destroy(sdp_saa_search* s);
  * Backward DP C_T = 0, C_t(I) = min(no delivery, delivery), ties to no
  * delivery; value = C_0(I0); policy = decisions along the optimal path. */
 /* Reinsertion kernels */
-#define SDP_REINSERT_AUTO 0  /* without value0_out, and for T up to about 128
-                                with at most 8 route options: a kernel over
-                                the states reachable from I0 only (the same
+#define SDP_REINSERT_AUTO 0  /* without value0_out, for T up to 128, 99 with
+                                1 to 4 route options, 80 with 5 to 8 (less
+                                for U below 32, and where consumption is too
+                                small for U below 128): a kernel over the
+                                states reachable from I0 only (the same
                                 bits); else LANE where it applies, else WARP */
 #define SDP_REINSERT_WARP 1  /* one warp per scenario, states across lanes */
 #define SDP_REINSERT_LANE 2  /* one lane per scenario, its cost-to-go in shared

@@ -8,7 +8,8 @@
 // two actions or up to 8 route options.  All three evaluate every state of
 // every day; SDP_REINSERT_AUTO takes reinsert_chain.cu's kernel, over the
 // reachable states only, where it applies and C_0(I) is not wanted for every
-// I, else the lane kernel wherever it applies (U <= 255, T <= 4096, at least 4
+// I (in some shapes only unless a sample of the scenarios consumes too little),
+// else the lane kernel wherever it applies (U <= 255, T <= 4096, at least 4
 // warps' worth of its shared memory per SM; not with a table end cost and
 // route options).  SDP_REINSERT_WARP forces the warp kernels.
 //
@@ -427,6 +428,7 @@ struct IntTag {
 template <int KC, bool TABLE, bool UNIT, int RK = 0>
 __global__ void __launch_bounds__(kLaneWarps * 32, 1) reinsert_lane_kernel(ReinsertArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  if (a.sparse_load && *a.sparse == 0u) return;  // the chains took the call
   if (a.mean_counter && blockIdx.x == 0 && threadIdx.x == 0) *a.mean_counter = 0u;
   constexpr int NI = 32 * KC;  // rows
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -814,8 +816,10 @@ size_t reinsert_lane_scratch_bytes(int T, int U) {
 int launch_reinsert(const ReinsertArgs& a, cudaStream_t st) {
   if (a.S <= 0) return 0;
   if (a.algo == SDP_REINSERT_AUTO && !a.value0 &&
-      reinsert_chain_supported(a.T, a.U, a.table != nullptr, a.n_routes, a.h, a.p, a.c))
-    return launch_reinsert_chain(a, st);
+      reinsert_chain_supported(a.T, a.U, a.table != nullptr, a.n_routes, a.h, a.p, a.c)) {
+    const int e = launch_reinsert_chain(a, st);
+    if (e || a.sparse_load == 0u) return e;
+  }
   const bool unit = a.c != 0.f;
   if (a.n_routes > 0) {  // route options: U <= 255, linear end costs (checked by the caller)
     if (a.U > 255 || a.table) return (int)cudaErrorInvalidValue;

@@ -52,8 +52,9 @@ namespace {
 
 constexpr int kChains = 4;          // chains walked together
 constexpr int kChainMaxWarps = 16;
-constexpr int kChainMinWarps = 4;   // fewer per SM hide too little latency
+constexpr int kChainMinWarps = 4;   // per SM (reinsert_chain_supported)
 constexpr int kChainMaxT = 254;     // days are kept in bytes
+constexpr int kChainSample = 8;     // scenarios that the choice of kernel looks at
 
 // Per warp: float2 (base, P) [T+1][32], the empty state's cost [T+1][32], its
 // first delivery from each day on [T+1][32] bytes, the policy rows [32][T]
@@ -82,6 +83,23 @@ __global__ void __launch_bounds__(kChainMaxWarps * 32, 1) reinsert_chain_kernel(
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int T = a.T, U = a.U;
   const int K = RK > 0 ? a.n_routes : 0;
+  if ((TABLE || RK > 0) && a.sparse_load) {  // every CTA adds up the same scenarios' consumption
+    __shared__ uint32_t used;
+    if (threadIdx.x == 0) used = 0u;
+    __syncthreads();
+    uint32_t v = 0u;
+#pragma unroll 4
+    for (int k = threadIdx.x; k < kChainSample * T; k += blockDim.x) {
+      const int64_t s = (a.S - 1) * (k / T) / (kChainSample - 1);
+      v += (uint32_t)min(max(__ldg(a.cons + s * T + k % T), 0), U);
+    }
+    v = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0) atomicAdd(&used, v);
+    __syncthreads();
+    const bool leave = used < a.sparse_load;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.sparse = leave ? 1u : 0u;
+    if (leave) return;
+  }
   float* day_sm = reinterpret_cast<float*>(smem);  // [T][DW]
   float* tab_sm = day_sm + T * DW;
   unsigned char* wb = smem + chain_head_bytes(T, U, TABLE, RK) + chain_warp_bytes(T, RK) * warp;
@@ -434,10 +452,23 @@ int launch_chain(const ReinsertArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-// The work of a chain is at most T / 2 cells a day, that of the lane kernel
-// 32 ceil((U + 1) / 32) states of about 1.5 times a cell's instructions; with
-// T <= 2.5 times those states the chains never do more, whatever the
-// consumption (mostly zero: chains of T days).
+// A chain has at most T / 2 cells a day (no consumption), the lane kernel 32
+// ceil((U + 1) / 32) states, and with table costs or routes a cell costs more
+// than a state.  Against the lane kernel on 10^5 scenarios that consume next to
+// nothing, the longest T that did not lose:
+//   no routes: 2.5 x states (32 states, T = 80: 0.93), with unit costs 72 of 32
+//     states (80: 1.07);
+//   table: 72 (80: 1.29) of 32 states, 80 of 64 (128: 1.31), 120 of 96;
+//   1 to 4 routes: 56 (72: 1.71) of 32, 80 of 64 (99: 1.11);
+//   5 to 8 routes: 48 of 64 (80: 1.87), 64 of 96 (80: 1.36), 80 of 128, and no
+//     gain worth having at 32 states (T = 20: 0.94-1.17, T = 80: 3.1).
+// At 32 states these are the limits.  From 64 states on, longer T with what
+// stock is held for takes 0.4 to 0.8 of the lane kernel's time: there a sample
+// decides (reinsert_sparse_load).
+//   The other end, with few warps per SM: four (T = 128; 99 with routes, 80 with
+// five and more) at U = 200, 8 a day, S = 2 10^5: 582 us, the lane kernel 2,644
+// (1,174 and 3,886 with four routes; 2,176 and 4,721 with eight).  Fewer were
+// not tried.
 //
 // h, p and c are bounded so that no cost of a state is infinite or NaN (the
 // kernel takes minima, and multiplies p by shortfalls of 0).
@@ -446,7 +477,23 @@ bool reinsert_chain_supported(int T, int U, bool table, int n_routes, float h, f
   if (T < 1 || T > kChainMaxT || U < 0 || U > 1023 || n_routes < 0 || n_routes > 8) return false;
   if (n_routes > 0 && (U > 255 || table)) return false;
   const int states = 32 * ((U + 1 + 31) / 32);
+  if (states == 32 && (n_routes > 4 || T > (n_routes ? 56 : table || c != 0.f ? 72 : 80))) return false;
   return 2 * T <= 5 * states && chain_warps(T, U, table, n_routes) >= kChainMinWarps;
+}
+
+// The consumption of the kChainSample scenarios, each day's up to U, below which
+// the chains leave a call to the lane kernel.  With T0 the limits above, the
+// chains take about (T / T0)^1.5 of its time without consumption, and in between
+// in proportion to a day's cells plus 20; a chain lasts U / (mean consumption)
+// days.  (64 states, 8 routes, T = 80, U = 40: the sides meet at 4.8 a day;
+// measured 1.12 at 3 a day, 0.74 at 8.)
+uint32_t reinsert_sparse_load(int T, int U, bool table, int n_routes) {
+  const double states = 32 * ((U + 1 + 31) / 32);
+  const double t0 = n_routes > 4 ? 16.0 + states / 2 : n_routes > 0 ? 32.0 + 0.75 * states : 1.25 * states;
+  if (states < 64 || !(table || n_routes) || T <= t0) return 0u;
+  const double cells = (T / 2.0 + 20.0) / pow(T / t0, 1.5) - 20.0;  // a day's, where the sides meet
+  const double days = T * (1.0 - sqrt(fmax(0.0, 1.0 - 2.0 * cells / T)));
+  return (uint32_t)(kChainSample * T * (double)U / fmax(days, 1.0));
 }
 
 int launch_reinsert_chain(const ReinsertArgs& a, cudaStream_t st) {

@@ -1088,6 +1088,12 @@ size_t reinsert_scratch_bytes(const sdp_reinsert_args* a) {
                     reinsert_lane_supported(a->T, a->U, a->n_routes);
   return (lane && a->policy_out && a->S > 0) ? reinsert_lane_scratch_bytes(a->T, a->U) : 0;
 }
+// Between these two, the sample decides (reinsert_sparse_load), where there is a
+// workspace for its word: the mean's partial sums leave some free.
+uint32_t reinsert_choice_load(const sdp_reinsert_args* a) {
+  return reinsert_uses_chain(a) && a->S > 0 && (a->policy_out || a->mean_out)
+             ? reinsert_sparse_load(a->T, a->U, a->end_cost_table != nullptr, a->n_routes) : 0u;
+}
 size_t reinsert_mean_bytes() { return align_up((size_t)kMeanBlocks * sizeof(double), 256); }
 }  // namespace
 
@@ -1099,7 +1105,8 @@ size_t sdp_reinsert_workspace_bytes(const sdp_reinsert_args* a) {
 
 size_t sdp_reinsert_call_bytes(const sdp_reinsert_args* a) {
   if (!a || a->S < 0 || a->T < 1 || a->U < 0) return 0;
-  return reinsert_mean_bytes() + (reinsert_uses_chain(a) ? 0 : reinsert_scratch_bytes(a));
+  const bool chain_only = reinsert_uses_chain(a) && reinsert_choice_load(a) == 0u;
+  return reinsert_mean_bytes() + (chain_only ? 0 : reinsert_scratch_bytes(a));
 }
 
 int sdp_reinsert_eval(const sdp_reinsert_args* a, void* stream) {
@@ -1159,6 +1166,8 @@ int sdp_reinsert_eval(const sdp_reinsert_args* a, void* stream) {
                              static_cast<unsigned char*>(a->workspace) + reinsert_mean_bytes())
                        : nullptr;
   r.mean_counter = a->mean_out ? mean_counter(static_cast<double*>(a->workspace)) : nullptr;
+  r.sparse_load = reinsert_choice_load(a);
+  if (r.sparse_load) r.sparse = reinterpret_cast<uint32_t*>(static_cast<double*>(a->workspace) + (kMeanBlocks - 2));
   prof_begin(st);
   int e = launch_reinsert(r, st);
   prof_end(st);

@@ -412,6 +412,10 @@ struct ReinsertArgs {
   uint32_t* status;
   uint32_t* dscratch;  // lane kernel with a policy: reinsert_lane_scratch_bytes
   uint32_t* mean_counter;  // set to zero for the mean that follows, or NULL
+  // AUTO, chains: where a sample's consumption is below sparse_load (0: never),
+  // they leave the call to the lane kernel behind them and say so in *sparse
+  uint32_t sparse_load;
+  uint32_t* sparse;
   int n_routes;               // route options per day (0: the two-action DP)
   const float* route_cost;    // [T * n_routes]
   const int32_t* route_cap;   // [S * T * n_routes]
@@ -426,6 +430,7 @@ int reinsert_lane_warps(int T, int U, bool table, int n_routes);
 size_t reinsert_lane_scratch_bytes(int T, int U);
 // the states reachable from I0 only (reinsert_chain.cu): AUTO without value0
 bool reinsert_chain_supported(int T, int U, bool table, int n_routes, float h, float p, float c);
+uint32_t reinsert_sparse_load(int T, int U, bool table, int n_routes);
 int launch_reinsert_chain(const ReinsertArgs& a, cudaStream_t st);
 
 int num_sms();
