@@ -55,6 +55,7 @@ constexpr int kChainMaxWarps = 16;
 constexpr int kChainMinWarps = 4;   // per SM (reinsert_chain_supported)
 constexpr int kChainMaxT = 254;     // days are kept in bytes
 constexpr int kChainSample = 8;     // scenarios that the choice of kernel looks at
+constexpr size_t kChainSmem = 227 * 1024 - 64;  // dynamic shared memory of a CTA, less the kernel's own
 
 // Per warp: float2 (base, P) [T+1][32], the empty state's cost [T+1][32], its
 // first delivery from each day on [T+1][32] bytes, the policy rows [32][T]
@@ -431,7 +432,7 @@ int chain_rk(int n_routes) { return n_routes == 0 ? 0 : n_routes <= 4 ? 4 : 8; }
 int chain_warps(int T, int U, bool table, int n_routes) {
   const int rk = chain_rk(n_routes);
   int w = kChainMaxWarps;
-  while (w > 0 && chain_head_bytes(T, U, table, rk) + chain_warp_bytes(T, rk) * w > 227 * 1024) --w;
+  while (w > 0 && chain_head_bytes(T, U, table, rk) + chain_warp_bytes(T, rk) * w > kChainSmem) --w;
   return w;
 }
 
