@@ -31,14 +31,19 @@
 // What bounds it: the fixed latencies of a cell's dependent operations with
 // 8 warps per SM (14 bytes of shared memory per scenario-day).  At T = 60,
 // U = 200, mean consumption 8, S = 10^6: 230 warp instructions per day and 32
-// scenarios against about 2,100 for the lane kernel; 0.65 ms, the lane kernel
-// 5.20 ms.  Four routes: 2.22 ms against 9.9.  Loading a day's record while
+// scenarios against about 2,100 for the lane kernel; 0.64 ms, the lane kernel
+// 5.20 ms.  Four routes: 2.11 ms against 9.9.  Loading a day's record while
 // the day above runs gave 5% of that (routes 1%), the L2 prefetch of the next
 // tile's rows 4% (3%).  11 warps per SM (16-bit prefix sums, decisions as bits)
 // took 263 instructions a day and the same time.  One chain at a time with
 // loops of each lane's own length took 1.14 ms (the decisions recorded in
 // every cell); two chains the same.
 //
+// Tiles with a daily cost below zero, or a day that consumes 2^24 / (T + 1) or
+// more, take tests that the others do without (ChainTile::days<true>, out of
+// line).  In long horizons of little consumption that is the slower way: with
+// costs below zero up to 1.7 of the lane kernel's time (U = 40, T = 120, one a
+// day), with such days 3.6; at U = 200, T = 60 0.9.
 #include <math.h>
 #include <math_constants.h>
 
@@ -69,10 +74,205 @@ __host__ __device__ constexpr size_t chain_head_bytes(int T, int U, bool table, 
   return (((size_t)T * (rk ? rk : 1) + (table ? U + 1 : 0)) * 4 + 15) & ~(size_t)15;
 }
 
-template <bool V>
-struct Flag {
-  static constexpr bool value = V;
+// A tile's chains: pointers are the lane's own (shared rows are strided by 32).
+template <bool TABLE, bool UNIT, int RK>
+struct ChainTile {
+  static constexpr int CW = RK / 4;            // capacity words per scenario-day
+  static constexpr int DW = RK > 0 ? RK : 1;   // daily costs per day
+  int T, lane;
+  float h, p, np, c, fU, e0;
+  int dmax;                // consumptions enter the prefix sums up to dmax
+  bool negc;               // some daily cost is negative
+  const float* day_sm;     // [T][DW]
+  const float* tab_sm;
+  float2* bp;              // (base, P) [s * 32]
+  float* zs;               // the empty state's cost [s * 32]
+  unsigned char* nz;       // its first delivery [s * 32]
+  unsigned char* pol;      // the warp's room for the policy
+  const uint32_t* cap;     // [(w T + s) * 32]
+  const int32_t* crow;     // the scenario's consumption
+  float zc, zn;            // C_{t+1}(0); what `left` adds: C, or e(0) + C in linear mode
+  int zfirst;
+
+  // the routes of a day: costs, and capacities as floats 2^23 + capacity (a
+  // byte under the exponent 0x4B)
+  struct Routes {
+    float cost[DW], cap[DW];
+  };
+  __device__ __forceinline__ Routes routes_of(int s) const {
+    Routes r;
+#pragma unroll
+    for (int w = 0; w < CW; ++w) {
+      const uint32_t cw = cap[(w * T + s) * 32];
+      const float4 rc = *reinterpret_cast<const float4*>(day_sm + s * DW + 4 * w);
+      const float cs[4] = {rc.x, rc.y, rc.z, rc.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        r.cost[(4 * w + e) % DW] = cs[e];
+        r.cap[(4 * w + e) % DW] = __uint_as_float(__byte_perm(cw, 0x4B000000u, 0x7540u | e));
+      }
+    }
+    return r;
+  }
+  // the delivery's value from state I of a day (v: its base): the cheapest
+  // route that carries U - I, +inf when none does
+  __device__ __forceinline__ float deliver(const Routes& r, float v, float I) const {
+    float dv = v;
+    if (RK > 0) {
+      const float qm = __fsub_rn(fU + 8388608.f, I);
+      float F = CUDART_INF_F;
+#pragma unroll
+      for (int k = 0; k < RK; ++k)
+        if (qm <= r.cap[k]) F = fminf(F, r.cost[k]);
+      dv = __fadd_rn(F, v);
+    }
+    if (UNIT) dv = __fadd_rn(dv, __fmul_rn(c, __fsub_rn(fU, I)));
+    return dv;
+  }
+  // nd of the day before day s >= 1, whose state x = A - P(s) this is: e(x)
+  // + C for x > 0; below, the stockout's cost on the empty state's zv.
+  // far (EXACT): what day s - 1 consumes if that is dmax or more, else 0; it is
+  // taken as it stands where the chain was still running on it, which is where
+  // this nd is used.
+  template <bool EXACT>
+  __device__ __forceinline__ float left(float A, float x, float C, float zv, int s, int far) const {
+    const bool on = x > 0.f;
+    if (TABLE) return __fadd_rn(tab_sm[max((int)x, 0)], on ? C : zv);
+    float m = x;
+    if (EXACT && far > 0 && !on)
+      m = -(float)(far - (int)fmaxf(__fsub_rn(A, bp[(s - 1) * 32].y), 0.f));
+    return __fadd_rn(__fmul_rn(on ? h : np, m), on ? C : zv);
+  }
+  // what day s - 1 consumes if that is dmax or more (of a day that mark() marked)
+  __device__ __forceinline__ int beyond(int s) const {
+    if (TABLE || !pol[s - 1] || __fsub_rn(bp[s * 32].y, bp[(s - 1) * 32].y) < (float)dmax) return 0;
+    return __ldg(crow + s - 1);
+  }
+  // the days on which some lane consumes dmax or more, in the policy's room
+  __device__ __forceinline__ void mark() {
+    for (int t = 0; t < T; ++t) {
+      const bool any = __any_sync(0xffffffffu, __fsub_rn(bp[(t + 1) * 32].y, bp[t * 32].y) >= (float)dmax);
+      if (lane == 0) pol[t] = any;
+    }
+    __syncwarp();
+  }
+
+  // day s of a chain at (A, nd); JOIN: it may still be empty
+  template <bool SLOW, bool JOIN>
+  __device__ __forceinline__ void cell(int s, float2 v, const Routes& r, float z, int far, float A, float& nd) const {
+    const float I = __fsub_rn(A, v.y);
+    const float dv = deliver(r, v.x, I);
+    float C;
+    if (SLOW) C = dv < nd && (!negc || I < fU) ? dv : nd;
+    else if (TABLE) C = dv < nd ? dv : nd;
+    else C = fminf(dv, nd);
+    if (JOIN) nd = left<SLOW>(A, I, C, z, s, far);
+    else nd = __fadd_rn(TABLE ? tab_sm[(int)I] : __fmul_rn(h, I), C);
+  }
+  // day s of the four chains
+  template <bool SLOW, bool JOIN>
+  __device__ __forceinline__ void cells(int s, float2 v, float z, const float* A, float* nd) const {
+    const Routes r = routes_of(s);
+    const int far = SLOW && JOIN ? beyond(s) : 0;
+#pragma unroll
+    for (int j = 0; j < kChains; ++j) cell<SLOW, JOIN>(s, v, r, z, far, A[j], nd[j]);
+  }
+
+  // All the days of the tile.  SLOW: some daily cost is negative or some
+  // consumption above dmax; otherwise no state equal to U gains by a delivery of
+  // nothing, and stockouts are the prefix loads' own.  (The minimum is an FMNMX:
+  // with h, p and c bounded, nd is never NaN, and a NaN delivery is not chosen
+  // either way.)
+  template <bool SLOW>
+  __device__ __forceinline__ void days() {
+    if (SLOW) mark();
+    // all chains of the warp are empty from day zhi on (or zhi = T), and
+    // all four are running from day zlo - 1 down (both only fall)
+    int zhi = T, zlo = T;
+    for (int t = T - 1; t >= 0; t -= kChains) {
+      float A[kChains], P[kChains], nd[kChains];
+#pragma unroll
+      for (int j = 0; j < kChains; ++j) {
+        P[j] = bp[max(t - j, 0) * 32].y;
+        A[j] = __fadd_rn(fU, P[j]);
+      }
+      while (zhi - 1 > t && !__any_sync(0xffffffffu, A[0] > bp[(zhi - 1) * 32].y)) --zhi;
+      zlo = min(zlo, zhi);
+      while (zlo - 1 > t && !__all_sync(0xffffffffu, A[kChains - 1] > bp[(zlo - 1) * 32].y)) --zlo;
+      {
+        const float Pz = bp[zhi * 32].y, z = zs[zhi * 32];
+        const int far = SLOW ? beyond(zhi) : 0;
+#pragma unroll
+        for (int j = 0; j < kChains; ++j)
+          nd[j] = left<SLOW>(A[j], __fsub_rn(A[j], Pz), -0.f, z, zhi, far);
+      }
+      // the next day's record is loaded while this day's cells run
+      int s = zhi - 1;
+      float2 v = bp[max(s, 0) * 32];
+#pragma unroll 1
+      for (; s >= zlo; --s) {
+        const float2 vn = bp[max(s - 1, 0) * 32];
+        cells<SLOW, true>(s, v, zs[s * 32], A, nd);
+        v = vn;
+      }
+#pragma unroll 4
+      for (; s > t; --s) {
+        const float2 vn = bp[max(s - 1, 0) * 32];
+        cells<SLOW, false>(s, v, 0.f, A, nd);
+        v = vn;
+      }
+      // days t .. t - 3: each chain comes down to its day, which gives that
+      // day's base and empty state, and the chains below take the day
+      float Pn = bp[(t + 1) * 32].y;
+#pragma unroll
+      for (int j = 0; j < kChains; ++j) {
+        const int d0 = t - j;
+        if (d0 < 0) break;
+        const float base = RK > 0 ? nd[j] : __fadd_rn(day_sm[d0], nd[j]);
+        float d = __fsub_rn(Pn, P[j]);
+        Pn = P[j];
+        if (SLOW && d >= (float)dmax) d = (float)max(__ldg(crow + d0), 0);
+        const Routes r = routes_of(d0);
+        const float G0 = TABLE ? __fadd_rn(e0, zc) : zn;
+        const float n0 = (TABLE || d == 0.f) ? G0 : __fadd_rn(G0, __fmul_rn(p, d));
+        const float dv = deliver(r, base, 0.f);
+        const bool dec = fU > 0.f && dv < n0;
+        zc = dec ? dv : n0;
+        zfirst = dec ? d0 : zfirst;
+        nz[d0 * 32] = (unsigned char)zfirst;
+        zn = TABLE ? zc : __fadd_rn(e0, zc);
+        bp[d0 * 32].x = base;
+        zs[d0 * 32] = zn;
+        if (d0 > 0) {
+          const int far = SLOW ? beyond(d0) : 0;
+#pragma unroll
+          for (int k = j + 1; k < kChains; ++k)
+            cell<SLOW, true>(d0, make_float2(base, P[j]), r, zn, far, A[k], nd[k]);
+        }
+      }
+    }
+    if (SLOW) __syncwarp();  // the marks are read before the policy takes their room
+  }
 };
+
+// Out of line: inlined, the tests of the rare tiles cost the others 1.5% (5% with
+// four routes).  A copy keeps the members in registers, and pointers made from
+// the block's own array are known to be shared memory.
+template <bool TABLE, bool UNIT, int RK>
+__device__ __noinline__ float slow_days(const ChainTile<TABLE, UNIT, RK>& tile) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  auto at = [&](const void* q) -> unsigned char* { return smem + (smem_u32(q) - smem_u32(smem)); };
+  ChainTile<TABLE, UNIT, RK> t = tile;
+  t.day_sm = reinterpret_cast<const float*>(at(tile.day_sm));
+  t.tab_sm = reinterpret_cast<const float*>(at(tile.tab_sm));
+  t.bp = reinterpret_cast<float2*>(at(tile.bp));
+  t.zs = reinterpret_cast<float*>(at(tile.zs));
+  t.nz = at(tile.nz);
+  t.pol = at(tile.pol);
+  t.cap = reinterpret_cast<const uint32_t*>(at(tile.cap));
+  t.template days<true>();
+  return t.zc;
+}
 
 template <bool TABLE, bool UNIT, int RK>
 __global__ void __launch_bounds__(kChainMaxWarps * 32, 1) reinsert_chain_kernel(ReinsertArgs a) {
@@ -206,155 +406,24 @@ __global__ void __launch_bounds__(kChainMaxWarps * 32, 1) reinsert_chain_kernel(
           }
       }
     }
-    // the routes of a day: costs, and capacities as floats 2^23 + capacity (a
-    // byte under the exponent 0x4B)
-    struct Routes {
-      float cost[DW], cap[DW];
-    };
-    auto routes_of = [&](int s) -> Routes {
-      Routes r;
-#pragma unroll
-      for (int w = 0; w < CW; ++w) {
-        const uint32_t cw = cap[(w * T + s) * 32];
-        const float4 rc = *reinterpret_cast<const float4*>(day_sm + s * DW + 4 * w);
-        const float cs[4] = {rc.x, rc.y, rc.z, rc.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          r.cost[(4 * w + e) % DW] = cs[e];
-          r.cap[(4 * w + e) % DW] = __uint_as_float(__byte_perm(cw, 0x4B000000u, 0x7540u | e));
-        }
-      }
-      return r;
-    };
-    // the delivery's value from state I of a day (v: its base): the cheapest
-    // route that carries U - I, +inf when none does
-    auto deliver = [&](const Routes& r, float v, float I) -> float {
-      float dv = v;
-      if (RK > 0) {
-        const float qm = __fsub_rn(fU + 8388608.f, I);
-        float F = CUDART_INF_F;
-#pragma unroll
-        for (int k = 0; k < RK; ++k)
-          if (qm <= r.cap[k]) F = fminf(F, r.cost[k]);
-        dv = __fadd_rn(F, v);
-      }
-      if (UNIT) dv = __fadd_rn(dv, __fmul_rn(c, __fsub_rn(fU, I)));
-      return dv;
-    };
-    // nd of the day before day s >= 1, whose state x = A - P(s) this is: e(x)
-    // + C for x > 0; below, the stockout's cost on the empty state's zc.
-    // EXACT: a day that consumes more than dmax is taken as it stands.
-    auto left = [&](auto exact, float A, float x, float C, float zc, int s) -> float {
-      const bool on = x > 0.f;
-      if (TABLE) return __fadd_rn(tab_sm[max((int)x, 0)], on ? C : zc);
-      float m = x;
-      if (decltype(exact)::value && !on) {
-        const float Pp = bp[(s - 1) * 32].y;
-        const int d = max(__ldg(crow + s - 1), 0);
-        // A - Pp > 0 where this nd is used
-        if (d > dmax) m = -(float)(d - (int)fmaxf(__fsub_rn(A, Pp), 0.f));
-      }
-      return __fadd_rn(__fmul_rn(on ? h : np, m), on ? C : zc);
-    };
-    // All the days of the tile.  SLOW: some daily cost is negative or some
-    // consumption above dmax: every test in every cell; otherwise no state
-    // equal to U gains by a delivery of nothing, and sums are exact.  (The
-    // minimum is an FMNMX: with h, p and c bounded, nd is never NaN, and a
-    // NaN delivery is not chosen either way.)
-    float zc = -0.f, zn = 0.f;  // C_{t+1}(0); what `left` adds: C, or e(0) + C in linear mode
-    int zfirst = T;
-    auto days = [&](auto slow) {
-      constexpr bool SLOW = decltype(slow)::value;
-      // day s of a chain at (A, nd); JOIN: it may still be empty
-      auto cell = [&](auto join, int s, float2 v, const Routes& r, float z, float A, float& nd) {
-        constexpr bool JOIN = decltype(join)::value;
-        const float I = __fsub_rn(A, v.y);
-        const float dv = deliver(r, v.x, I);
-        float C;
-        if (SLOW) C = dv < nd && (!negc || I < fU) ? dv : nd;
-        else if (TABLE) C = dv < nd ? dv : nd;
-        else C = fminf(dv, nd);
-        if (JOIN) nd = left(Flag<SLOW>{}, A, I, C, z, s);
-        else nd = __fadd_rn(TABLE ? tab_sm[(int)I] : __fmul_rn(h, I), C);
-      };
-      // day s of the four chains
-      auto cells = [&](auto join, int s, float2 v, float z, const float* A, float* nd) {
-        const Routes r = routes_of(s);
-#pragma unroll
-        for (int j = 0; j < kChains; ++j) cell(join, s, v, r, z, A[j], nd[j]);
-      };
-      // all chains of the warp are empty from day zhi on (or zhi = T), and
-      // all four are running from day zlo - 1 down (both only fall)
-      int zhi = T, zlo = T;
-      for (int t = T - 1; t >= 0; t -= kChains) {
-        float A[kChains], P[kChains], nd[kChains];
-#pragma unroll
-        for (int j = 0; j < kChains; ++j) {
-          P[j] = bp[max(t - j, 0) * 32].y;
-          A[j] = __fadd_rn(fU, P[j]);
-        }
-        while (zhi - 1 > t && !__any_sync(0xffffffffu, A[0] > bp[(zhi - 1) * 32].y)) --zhi;
-        zlo = SLOW ? t + 1 : min(zlo, zhi);
-        while (zlo - 1 > t && !__all_sync(0xffffffffu, A[kChains - 1] > bp[(zlo - 1) * 32].y)) --zlo;
-        {
-          const float Pz = bp[zhi * 32].y, z = zs[zhi * 32];
-#pragma unroll
-          for (int j = 0; j < kChains; ++j)
-            nd[j] = left(Flag<SLOW>{}, A[j], __fsub_rn(A[j], Pz), -0.f, z, zhi);
-        }
-        // the next day's record is loaded while this day's cells run
-        int s = zhi - 1;
-        float2 v = bp[max(s, 0) * 32];
-#pragma unroll 1
-        for (; s >= zlo; --s) {
-          const float2 vn = bp[max(s - 1, 0) * 32];
-          cells(Flag<true>{}, s, v, zs[s * 32], A, nd);
-          v = vn;
-        }
-        if (!SLOW) {
-#pragma unroll 4
-          for (; s > t; --s) {
-            const float2 vn = bp[max(s - 1, 0) * 32];
-            cells(Flag<false>{}, s, v, 0.f, A, nd);
-            v = vn;
-          }
-        }
-        // days t .. t - 3: each chain comes down to its day, which gives that
-        // day's base and empty state, and the chains below take the day
-        float Pn = bp[(t + 1) * 32].y;
-#pragma unroll
-        for (int j = 0; j < kChains; ++j) {
-          const int d0 = t - j;
-          if (d0 < 0) break;
-          const float base = RK > 0 ? nd[j] : __fadd_rn(day_sm[d0], nd[j]);
-          float d = __fsub_rn(Pn, P[j]);
-          Pn = P[j];
-          if (SLOW) d = (float)max(__ldg(crow + d0), 0);
-          const Routes r = routes_of(d0);
-          const float G0 = TABLE ? __fadd_rn(e0, zc) : zn;
-          const float n0 = (TABLE || d == 0.f) ? G0 : __fadd_rn(G0, __fmul_rn(p, d));
-          const float dv = deliver(r, base, 0.f);
-          const bool dec = U > 0 && dv < n0;
-          zc = dec ? dv : n0;
-          zfirst = dec ? d0 : zfirst;
-          nz[d0 * 32] = (unsigned char)zfirst;
-          zn = TABLE ? zc : __fadd_rn(e0, zc);
-          bp[d0 * 32].x = base;
-          zs[d0 * 32] = zn;
-          if (d0 > 0) {
-#pragma unroll
-            for (int k = j + 1; k < kChains; ++k)
-              cell(Flag<true>{}, d0, make_float2(base, P[j]), r, zn, A[k], nd[k]);
-          }
-        }
-      }
-    };
-    zn = TABLE ? zc : __fadd_rn(e0, zc);
-    zs[T * 32] = zn;
+    ChainTile<TABLE, UNIT, RK> ct;
+    ct.T = T; ct.lane = lane;
+    ct.h = h; ct.p = p; ct.np = np; ct.c = c; ct.fU = fU; ct.e0 = e0;
+    ct.dmax = dmax; ct.negc = negc;
+    ct.day_sm = day_sm; ct.tab_sm = tab_sm;
+    ct.bp = bp; ct.zs = zs; ct.nz = nz; ct.pol = pol; ct.cap = cap; ct.crow = crow;
+    ct.zc = -0.f;
+    ct.zn = TABLE ? ct.zc : __fadd_rn(e0, ct.zc);
+    ct.zfirst = T;
+    zs[T * 32] = ct.zn;
     nz[T * 32] = (unsigned char)T;
     const bool slow = negc || __any_sync(0xffffffffu, big);
-    if (slow) days(Flag<true>{});
-    else days(Flag<false>{});
+    if (slow) {
+      const ChainTile<TABLE, UNIT, RK> copy = ct;
+      ct.zc = slow_days(copy);
+    } else {
+      ct.template days<false>();
+    }
 
     // ---- the path from I0.  Only a few chains are on it, so the days on
     // which a chain delivers are found by walking it again.
@@ -369,13 +438,14 @@ __global__ void __launch_bounds__(kChainMaxWarps * 32, 1) reinsert_chain_kernel(
       int first = nz[z * 32];
       if (z == t0) return first;
       const float x = __fsub_rn(A, bp[z * 32].y);
-      float nd = slow ? left(Flag<true>{}, A, x, -0.f, zs[z * 32], z)
-                      : left(Flag<false>{}, A, x, -0.f, zs[z * 32], z);
+      const int far = slow && !TABLE ? max(__ldg(crow + z - 1), 0) : 0;
+      float nd = slow ? ct.template left<true>(A, x, -0.f, zs[z * 32], z, far >= dmax ? far : 0)
+                      : ct.template left<false>(A, x, -0.f, zs[z * 32], z, 0);
 #pragma unroll 2
       for (int s = z - 1; s >= t0; --s) {
         const float2 v = bp[s * 32];
         const float I = __fsub_rn(A, v.y);
-        const float dv = deliver(routes_of(s), v.x, I);
+        const float dv = ct.deliver(ct.routes_of(s), v.x, I);
         const bool dec = dv < nd && (!negc || I < fU);
         C = dec ? dv : nd;
         if (dec) first = s;
@@ -383,7 +453,7 @@ __global__ void __launch_bounds__(kChainMaxWarps * 32, 1) reinsert_chain_kernel(
       }
       return first;
     };
-    float A = (float)a.I0, C = zc;
+    float A = (float)a.I0, C = ct.zc;
     int day = walk(A, 0, C);
     if (live) a.value[s0 + lane] = __fadd_rn(0.f, C);
     if (a.policy) {
