@@ -321,8 +321,8 @@ int sdp_split_backward(const sdp_split_args* fwd, const void* pred,
  * sdp_split_routes_workspace_bytes(a) is its workspace, 0 where it does not
  * run (SDP_ERR_UNSUPPORTED).  cost_out may be NULL (size the workspace with
  * the same cost_out as the call).  sdp_split_step_workspace_bytes(a) is the
- * same where this pass takes about the time of the evaluation alone (n <= 50,
- * or n <= 336 and all scenarios in one round of the kernel), else 0: what a
+ * same where this pass takes at most about one and a half times the evaluation
+ * alone (n <= 64, or up to 42 tiles of 32 scenarios per SM), else 0: what a
  * training step uses that cannot know whether its backward will be called.
  * sdp_split_grad_from_routes turns them into d mean / d dist [(n+1)^2] times
  * *grad_mean (a device float, or a double that is rounded to float first). */

@@ -466,10 +466,11 @@ class SplitMeanCost(torch.autograd.Function):
     forward(dist [n+1, n+1] fp32 CUDA, tour, demands, Q, keep_pred=False)
     returns the FP64 scenario mean (0-d); backward returns
     d mean / d dist = (1/S) x arc-usage counts of the optimal splits (the
-    cost is piecewise linear in dist).  Where a gradient is wanted, the fused
-    kernel applies and takes no longer than the evaluation alone, the forward
-    counts the routes while it evaluates and the backward only assembles the
-    matrix; otherwise the counts come
+    cost is piecewise linear in dist).  Where a gradient is wanted and the
+    fused kernel applies, the forward counts the routes while it evaluates and
+    the backward only assembles the matrix, up to about 200,000 scenarios (any
+    number for n <= 64): beyond, a forward without a backward would lose more
+    than it should, and for a mean alone turn gradients off.  Otherwise the counts come
     from stored predecessors (keep_pred=True) by the library's backtrack
     kernel or are recomputed by the fused forward + backtrack kernel."""
 
@@ -507,7 +508,7 @@ class SplitMeanCost(torch.autograd.Function):
 def _split_mean_routes(tour, Q, demands, dist):
     """split_eval's mean and the route counts int64 [2n + 1] of the optimal
     splits from one kernel; (None, None) where no kernel returns both, or the
-    mean alone takes less time."""
+    mean alone takes much less time."""
     lib = _load()
     n, dev = int(tour.numel()), tour.device
     a = _split_struct(tour, Q, demands, None, dist, None, None, 0, "auto", None, 0, 0)

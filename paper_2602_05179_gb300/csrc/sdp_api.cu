@@ -1000,21 +1000,25 @@ size_t sdp_split_routes_workspace_bytes(const sdp_split_args* a) {
   return carve_split(a, nullptr, true, false).bytes + (a->cost_out ? 0 : sizeof(float) * (size_t)a->S);
 }
 
-// The adjoint's kernel counts routes behind the recursion and runs 16 to 24
-// warps per SM, PIPE 23 without counting, so a forward whose backward never
-// comes pays for the counts.  Its time over the separate forward's (memset,
-// preparation, PIPE, recomputation, two kernels for the mean) was, with 3 to 24
-// customers a route:
-//   tiles in one round of the kernel: n = 32..200 0.61-1.06, n = 250..336
-//     0.90-1.13 (1.05 with 6 customers a route or more but for n = 250 at 21
-//     tiles per SM, 1.11), n = 500 1.03-1.13;
-//   more rounds: n = 32 0.51-0.75, n = 50 0.78-1.01, n = 64 0.81-1.11,
-//     n = 100 0.91-1.55, n = 300 1.36-2.03 (S = 2 10^5: 231 -> 334 us).
-// One pass serves both where it costs the forward (next to) nothing.
+// One pass saves the step a recursion (a third of it and more: n = 362, S = 32,137
+// 313 -> 230 us), but a forward whose backward never comes pays for the counts:
+// the adjoint's kernel counts routes behind the recursion, on 16 to 24 warps per
+// SM where PIPE has 23 and does not count.  Over the separate forward's time
+// (memset, preparation, PIPE, recomputation, two kernels for the mean), with 6
+// to 24 customers a route (3 a route: up to 0.15 more):
+//   tiles in one round of the kernel: n = 32..200 0.61-1.02, n = 250..336
+//     0.90-1.11, n = 420 0.97-1.05, n = 500 1.03-1.13;
+//   up to 42 tiles per SM: n = 100 0.91-1.03, n = 120 1.00-1.14, n = 183
+//     1.36-1.53, n = 300 1.36-1.53 (S = 2 10^5: 231 -> 334 us);
+//   more: n = 50 0.78-0.89, n = 64 0.81-0.96, n = 100 1.08-1.32, n = 183
+//     1.72-1.97, n = 300 1.56-1.83 (S = 10^6: 696 -> 1,186 us, the step 1,859 ->
+//     1,206).
+// So one pass serves both as long as what such a forward loses is a small part
+// of what the step gains; programs that want the mean alone run it with
+// gradients off, which is PIPE at every size.
 static bool routes_pay(const sdp_split_args* a) {
-  if (a->n <= 50) return true;
   const int64_t tiles = (a->S + 31) / 32;
-  return a->n <= 336 && tiles <= (int64_t)adjoint_tmem_warps(a, false) * num_sms();
+  return a->n <= 64 || tiles <= 42 * (int64_t)num_sms();
 }
 
 size_t sdp_split_step_workspace_bytes(const sdp_split_args* a) {

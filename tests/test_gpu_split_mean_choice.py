@@ -1,7 +1,6 @@
-"""When SplitMeanCost's forward counts the routes as it evaluates: in one round
-of the adjoint's kernel, where that costs a forward without a backward nothing,
-and for short tours; beyond, the forward is the evaluation alone.  Mean and
-gradient are the same bits on both sides of each line."""
+"""When SplitMeanCost's forward counts the routes as it evaluates: for tours up to
+64, and up to 42 tiles per SM; beyond, the forward is the evaluation alone.
+Mean and gradient are the same bits on both sides of each line."""
 import numpy as np
 import pytest
 
@@ -9,29 +8,23 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-def _round(n, Q):
-    """Scenarios of one round: as many warps per SM, 16 to 24, as have tensor
-    memory columns for a row (rows take a multiple of four)."""
-    words = ((n if Q <= 254 else 2 * n) + 15) // 16 * 4
-    warps = max(w for w in range(16, 25) if words <= (512 // ((w + 3) // 4) & ~3))
-    return 32 * warps * torch.cuda.get_device_properties(0).multi_processor_count
-
-
-@pytest.mark.parametrize("n,Q,over,fused", [
-    (50, 100, 40_000, True),
-    (51, 100, 0, True),
-    (51, 100, 1, False),
-    (100, 300, 0, True),
-    (100, 300, 1, False),
-    (200, 300, 0, True),      # rows of 400 bytes: 20 warps
-    (200, 300, 1, False),
-    (336, 100, 0, True),
-    (336, 100, 1, False),
-    (337, 100, -50_000, False),
+@pytest.mark.parametrize("n,Q,tiles,over,fused", [
+    (64, 100, 60, 0, True),
+    (65, 100, 42, 0, True),
+    (65, 100, 42, 1, False),
+    (120, 300, 42, 0, True),
+    (120, 300, 42, 1, False),
+    (200, 300, 20, 0, True),      # one round of 20 warps, and a second one begun
+    (200, 300, 20, 1, True),
+    (336, 100, 24, 1, True),
+    (500, 100, 42, 0, True),
+    (500, 100, 42, 1, False),
+    (513, 100, 1, 0, False),      # rows that the kernel does not hold
 ])
-def test_choice_and_bits(n, Q, over, fused):
+def test_choice_and_bits(n, Q, tiles, over, fused):
     from paper_2602_05179_gb300 import api
-    S = _round(n, Q) + over
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    S = 32 * tiles * sms + over
     rng = np.random.default_rng(n + Q)
     g = torch.Generator(device="cuda")
     g.manual_seed(n)
