@@ -11,7 +11,7 @@
 // psi_{k-1}(p) = K_{k-1}(p) + a_{p+1} -- the Split recursion fed by the layer
 // below -- and every layer has the same capacity window.
 //
-// split_fleet_band_kernel (AUTO up to n of about 1,700): one warp per
+// split_fleet_band_kernel (AUTO up to n = 1,855 to 1,879, by K): one warp per
 // scenario, layer after layer, over the band of positions that matter.  A
 // split into at most K routes passes (k, i) only if n can be reached from i
 // with K - k more routes, i >= lo_k, and i from 0 with k, i <= hi_k: both
@@ -19,8 +19,8 @@
 // the tour's end, hi from its start), every feasible p of a position in the
 // band lies in the band below, so the values in it are those of the full
 // recursion.  A binding fleet leaves few routes of slack, and the band is
-// slack routes wide: at n = 500, Q = 200, K = 42 (about 41 needed) some 26
-// positions of 500.  Within a layer the positions are independent: a lane
+// slack routes wide: at n = 500, Q = 200, K = 42 (about 41 needed) 19
+// positions of 500 on average.  Within a layer the positions are independent: a lane
 // each, windows by minima of blocks of B positions (built once per layer in
 // shared memory), values only.  The layers' psi rows go to a scratch of the
 // warp (band only, in L2), and the path is found from the last layer back,
