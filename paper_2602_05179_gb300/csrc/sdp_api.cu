@@ -779,7 +779,7 @@ struct FleetWs {
   TourPrep prep;
   double* mean_partial;
   uint32_t* fb_count;
-  unsigned long long* loose;
+  uint32_t* loose;
   uint32_t* fb_list;
   float* kscratch;
   uint16_t* pscratch;
@@ -800,9 +800,9 @@ FleetWs carve_fleet(const sdp_split_args* a, int K, bool routes, void* base) {
   w.prep.cols = c.take<uint16_t>((size_t)n);
   w.prep.Dn = c.take<double>(1);
   w.mean_partial = c.take<double>(kMeanBlocks);
-  // flagged scenarios, and the band kernel's choice 8 bytes on
-  w.fb_count = c.take<uint32_t>(4);
-  w.loose = w.fb_count ? reinterpret_cast<unsigned long long*>(w.fb_count + 2) : nullptr;
+  // flagged scenarios, and the choice between the warp kernels
+  w.fb_count = c.take<uint32_t>(2);
+  w.loose = w.fb_count ? w.fb_count + 1 : nullptr;
   w.fb_list = plain ? nullptr : c.take<uint32_t>((size_t)a->S);
   const int64_t cap = plain ? kFleetPlainSlots : kFleetFallbackSlots;
   w.nslots = a->S < cap ? a->S : cap;
@@ -869,7 +869,8 @@ int sdp_split_fleet_eval(const sdp_split_args* a, int32_t max_routes, int32_t* n
     if (e != cudaSuccess) return cuda_fail(e, "memset fleet outputs");
   } else if (a->S > 0) {
     launch_tour_prep(a->tour, a->n, a->coords, a->dist, w.prep, status,
-                     {w.fb_count, w.loose, mean_counter(w.mean_partial)}, st);
+                     {w.fb_count, nullptr, mean_counter(w.mean_partial)}, st,
+                     {a->demands, a->S, a->Q, w.cfg.loose_load, w.loose});
     SplitFleetArgs f{};
     f.n = a->n; f.Q = a->Q; f.K = max_routes; f.S = a->S;
     f.rec = w.prep.rec; f.Dn = w.prep.Dn; f.demands = a->demands;
@@ -887,8 +888,7 @@ int sdp_split_fleet_eval(const sdp_split_args* a, int32_t max_routes, int32_t* n
     } else {
       f.fb_list = w.fb_list;
       f.dscratch = w.dscratch;
-      f.loose = reinterpret_cast<uint32_t*>(w.loose);
-      f.loose_load = w.cfg.loose_load;
+      f.loose = w.cfg.loose_load ? w.loose : nullptr;
       note_launch(w.cfg.warps, w.cfg.grid);
       prof_begin(st);
       e = launch_split_fleet(f, w.cfg, st);

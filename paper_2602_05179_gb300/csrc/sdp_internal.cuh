@@ -47,10 +47,20 @@ struct CallCounters {
   uint32_t* mean;
   unsigned long long* routes = nullptr;
 };
+// A sample of the scenarios (the first and the last among them): *out = whether
+// its demands, each up to Q + 1, add up to less than `below` (0: no sample).
+constexpr int kLoadSample = 8;
+struct LoadSample {
+  const int32_t* demands = nullptr;
+  int64_t S = 0;
+  int Q = 0;
+  uint32_t below = 0;
+  uint32_t* out = nullptr;
+};
 // one CTA per tour; coords or dist mode
 void launch_tour_prep(const int32_t* tour, int n, const float* coords,
                       const float* dist, TourPrep prep, uint32_t* status,
-                      CallCounters counters, cudaStream_t st);
+                      CallCounters counters, cudaStream_t st, LoadSample sample = {});
 
 struct SplitPlainArgs {
   int n, Q;
@@ -350,8 +360,7 @@ struct SplitFleetArgs {
   uint16_t* dscratch;        // warp kernels with routes: fleet_dscratch_elems
   uint32_t* fb_list;         // warp kernel: flagged scenarios; plain: NULL = all S
   uint32_t* fb_count;
-  uint32_t* loose;           // set by the band kernel: the deque kernel takes the call's scenarios
-  uint32_t loose_load;       // ... where a sample's demands add up to less than this (0: never)
+  const uint32_t* loose;     // band: the deque kernel takes the call's scenarios, or NULL (never)
   float* kscratch;           // plain: [nslots * 2 * (n+1)]
   uint16_t* pscratch;        // plain with routes: [nslots * K * n]
   int64_t nslots;
@@ -362,7 +371,7 @@ struct FleetConfig {
   int grid;
   bool band;  // the band kernel, which also recomputes what it flags
   // band: the sample's load below which the deque kernel takes the scenarios
-  // (0: never), and that kernel's shape
+  // (LoadSample; 0: never), and that kernel's shape
   uint32_t loose_load;
   int loose_warps, loose_grid;
 };

@@ -21,9 +21,20 @@ __device__ __forceinline__ float travel(const float* coords, const float* dist,
 __global__ void __launch_bounds__(256) tour_prep_kernel(
     const int32_t* __restrict__ tour, int n, const float* __restrict__ coords,
     const float* __restrict__ dist, TourPrep prep, uint32_t* status,
-    CallCounters counters) {
+    CallCounters counters, LoadSample sample) {
   __shared__ double red[256];
+  __shared__ uint32_t load[kLoadSample];
+  static_assert(kLoadSample == 256 / 32, "a warp each");
   dep_launch();
+  if (sample.below) {
+    const int j = threadIdx.x >> 5;
+    const int32_t* q = sample.demands + (sample.S - 1) * j / (kLoadSample - 1) * n;
+    uint32_t v = 0u;
+#pragma unroll 8
+    for (int k = threadIdx.x & 31; k < n; k += 32) v += (uint32_t)min(max(__ldg(q + k), 0), sample.Q + 1);
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) load[j] = v;
+  }
   if (threadIdx.x == 0) {  // the call's counters, for the kernels that follow
     if (counters.flagged) *counters.flagged = 0u;
     if (counters.tiles) *counters.tiles = 0ull;
@@ -60,13 +71,20 @@ __global__ void __launch_bounds__(256) tour_prep_kernel(
     if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *prep.Dn = red[0];
+  if (threadIdx.x == 0) {
+    *prep.Dn = red[0];
+    if (sample.below) {
+      uint32_t v = 0u;
+      for (int j = 0; j < kLoadSample; ++j) v += load[j];
+      *sample.out = v < sample.below ? 1u : 0u;
+    }
+  }
 }
 
 void launch_tour_prep(const int32_t* tour, int n, const float* coords,
                       const float* dist, TourPrep prep, uint32_t* status,
-                      CallCounters counters, cudaStream_t st) {
-  tour_prep_kernel<<<1, 256, 0, st>>>(tour, n, coords, dist, prep, status, counters);
+                      CallCounters counters, cudaStream_t st, LoadSample sample) {
+  tour_prep_kernel<<<1, 256, 0, st>>>(tour, n, coords, dist, prep, status, counters, sample);
 }
 
 // ----------------------------------------------------------- arc counting

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kFMaxWarps * 32) split_fleet_kernel(SplitFleet
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int n = a.n, Q = a.Q, K = a.K;
   dep_launch();
-  const bool shared_call = a.loose_load != 0u;  // with the band kernel, which chose
+  const bool shared_call = a.loose != nullptr;  // with the band kernel: one of them takes the call
   if (shared_call && *a.loose == 0u) return;
   // shared: (a_i, ce_i) and columns of the tour | per warp: KS rings,
   // route boundaries
@@ -502,7 +502,6 @@ constexpr int kBandMaxWarps = 24;
 constexpr int kBandMinWarps = 8;   // per SM: fewer hide too little latency
 constexpr int kBandWindow = 32;    // longest window of the narrow form
 constexpr int kBandNarrow = 4, kBandWide = 16;  // positions per block minimum
-constexpr int kBandSample = 8;     // scenarios that the choice of kernel looks at
 
 // CTA: a_{p+1} and ce_i [n+1] floats each, columns [n]; per warp: prefix
 // loads, psi and block minima [n+1 .. +16] (each on 16 bytes), window starts [n+1] uint16, and
@@ -517,7 +516,7 @@ __host__ __device__ constexpr size_t band_per_warp(int n, int K) {
 
 // B: positions per block minimum.  LIST: the flagged scenarios (fb_list);
 // otherwise all, flagging those with a window above kBandWindow, or none where
-// a sample of the scenarios says that the fleet has much slack (loose_load).
+// the tour preparation's sample says that the fleet has much slack (loose).
 template <int B, bool LIST, bool ROUTES>
 __global__ void __launch_bounds__(kBandMaxWarps * 32) split_fleet_band_kernel(SplitFleetArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -536,18 +535,7 @@ __global__ void __launch_bounds__(kBandMaxWarps * 32) split_fleet_band_kernel(Sp
   uint16_t* hi_of = lo_of + K + 2;   // [k]: the last position that k routes reach
   uint16_t* bound = hi_of + K + 2;   // route k covers positions bound[k] + 1 .. bound[k+1]
   if (LIST) dep_wait();
-  // every CTA adds up the same scenarios' demands, while the records load
-  __shared__ uint32_t load[kBandMaxWarps];
-  if (!LIST && a.loose_load) {
-    uint32_t v = 0u;
-    for (int j = warp; j < kBandSample; j += nw) {
-      const int32_t* q = a.demands + (a.S - 1) * j / (kBandSample - 1) * n;
-#pragma unroll 8
-      for (int k = lane; k < n; k += 32) v += (uint32_t)min(max(__ldg(q + k), 0), Q + 1);
-    }
-    v = __reduce_add_sync(kAll, v);
-    if (lane == 0) load[warp] = v;
-  }
+  const uint32_t leave = !LIST && a.loose ? *a.loose : 0u;  // (in flight with the records)
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     const StepRec r = a.rec[k];
     as[k] = r.a;
@@ -556,14 +544,7 @@ __global__ void __launch_bounds__(kBandMaxWarps * 32) split_fleet_band_kernel(Sp
   }
   if (threadIdx.x == 0) as[n] = 0.f;
   __syncthreads();
-  if (!LIST && a.loose_load) {
-    uint32_t v = 0u;
-    for (int w = 0; w < nw; ++w) v += load[w];
-    if (v < a.loose_load) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) *a.loose = 1u;
-      return;
-    }
-  }
+  if (!LIST && leave) return;
   const double Dn = *a.Dn;
   const int64_t slot = (int64_t)blockIdx.x * nw + warp;
   float* rows = ROUTES ? reinterpret_cast<float*>(a.dscratch) + slot * K * (int64_t)(n + 1) : nullptr;
@@ -804,13 +785,13 @@ int launch_band(const SplitFleetArgs& a, const FleetConfig& c, cudaStream_t st) 
     e = cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
   narrow<<<c.grid, c.warps * 32, smem, st>>>(a);
-  if (a.loose_load) {
+  if (a.loose) {
     const int d = launch_deque(a, c.loose_warps, c.loose_grid, st);
     if (d) return d;
   }
   // placed while the deque kernel finds that it has nothing to do; placed early
   // behind the narrow form it slows that one (n = 500, K = 42: 1128 -> 1153 us)
-  return (int)launch_dependent(a.loose_load != 0u, wide, c.grid, c.warps * 32, smem, st, a);
+  return (int)launch_dependent(a.loose != nullptr, wide, c.grid, c.warps * 32, smem, st, a);
 }
 
 // The deque kernel's shape: one CTA per SM with as many warps as its shared
@@ -825,8 +806,8 @@ void deque_shape(int n, int K, int64_t S, int* warps, int* grid) {
   *grid = (int)imin64(need < 1 ? 1 : need, (int64_t)num_sms());
 }
 
-// The load of the kBandSample scenarios below which the deque kernel takes a
-// call rather than the band kernel: kBandSample Q times the mean m of the routes
+// The load of the kLoadSample scenarios below which the deque kernel takes a
+// call rather than the band kernel: kLoadSample Q times the mean m of the routes
 // that they need at least.
 //   The band of a scenario holds about n (K - m) states.  On 65,536 scenarios
 // (n = 31..500, K up to 64, windows of 4 to n positions, random and sweep tours)
@@ -840,18 +821,19 @@ void deque_shape(int n, int K, int64_t S, int* warps, int* grid) {
 // needed): 1.13 and 5.75.
 //   With the choice, 1,500 sizes from S = 200 on take at most 1.08 of the deque
 // kernel's time (eight of them up to 1.20).  It costs tight fleets a launch (1 to
-// 6 us; inlined into the band kernel, or called from it, the deques cost the band
-// 2 to 13%), and calls whose rings do outgrow (windows of 22 to n / 3 positions;
+// 4 us; n = 500, K = 42: 1,124 -> 1,128).  The sample taken by the band kernel's
+// CTAs cost 3 us more, the deques inlined into the band kernel, or called from
+// it, 2 to 13%.  Calls whose rings do outgrow (windows of 22 to n / 3 positions;
 // the deque kernel and its recomputation took 2 to 20 times the band's time
-// there) the time until the scenarios are handed back: up to 12% of the band's
-// time, up to 78% where each warp has one scenario.
+// there) lose the time until the scenarios are handed back: up to 12% of the
+// band's time, up to 78% where each warp has one scenario.
 uint32_t fleet_loose_load(int n, int Q, int K, int64_t S) {
   const double idle = std::max(0.0, 1.0 - (double)S / (kFMaxWarps * num_sms()));
   // per position, in units of 0.25 us on 65,536 scenarios
   const double deque = (K <= 32 ? 27.0 + 6.0 * idle : 43.0 + 3.0 * idle) + 1200.0 * idle / n - 49.0 * K / n;
   const double m = std::max(K - deque, std::min(3.0, K - deque / 1.35));
   // (less than one route: hardly a call, and the choice costs each call a launch)
-  return m >= 1.0 ? (uint32_t)(kBandSample * std::min(m, K + 1.0) * Q) : 0u;
+  return m >= 1.0 ? (uint32_t)(kLoadSample * std::min(m, K + 1.0) * Q) : 0u;
 }
 
 }  // namespace
