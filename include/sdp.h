@@ -503,7 +503,7 @@ void sdp_saa_search_destroy(sdp_saa_search* s);
 #define SDP_REINSERT_AUTO 0  /* without value0_out, for T up to 128, 99 with
                                 1 to 4 route options, 80 with 5 to 8 (less
                                 for U below 32, and where consumption is too
-                                small for U below 128): a kernel over the
+                                small for U below 96): a kernel over the
                                 states reachable from I0 only (the same
                                 bits); else LANE where it applies, else WARP */
 #define SDP_REINSERT_WARP 1  /* one warp per scenario, states across lanes */

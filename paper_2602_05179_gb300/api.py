@@ -528,7 +528,8 @@ def _grad_from_routes(tour, S, routes, grad_mean):
     """d mean / d dist (fp32 [n+1, n+1]) times grad_mean from route counts."""
     n = int(tour.numel())
     grad = torch.empty((n + 1, n + 1), dtype=torch.float32, device=tour.device)
-    gm = grad_mean.resolve_neg()  # its memory is read: a lazily negated one holds the other sign
+    # its memory is read: a lazily negated one holds the other sign
+    gm = grad_mean.resolve_neg() if grad_mean.is_neg() else grad_mean
     if gm.device != tour.device or gm.dtype not in (torch.float32, torch.float64):
         gm = gm.to(device=tour.device, dtype=torch.float32)
     # a saved-tensor hook may have put other tensors in the place of these two
